@@ -215,9 +215,10 @@ void silu_mat_destroy(silu_mat A);
  * 10: the narrow configuration -- tiles of at most 352 entries swept by 24
  * warps per SM with 10 gathers in flight, for one lane and one row per lane
  * and rows of at most 10 entries, 9 on average, else SILU_ERR_INVALID_ARG;
- * 0: automatic, the narrow configuration where it fits, else 16).  The
- * automatic shape (lanes 0, passes 0, chunk 0) is what silu_mat_create
- * chooses.  Results change only by summation order across lanes.  Blocks (the new
+ * 0: automatic, the narrow configuration where it fits, else 16).  Lanes 0,
+ * passes 0, chunk 0 is what silu_mat_create chooses: the sliced kernel where
+ * A has a sliced copy (see silu_ilu_set_kernel), else the staged kernel in
+ * its automatic shape, with the same bits for one right-hand side.  Results change only by summation order across lanes.  Blocks (the new
  * tiles are uploaded); captured FGMRES iterations of factor objects on A are
  * rebuilt on their next use.
  */
@@ -226,7 +227,8 @@ silu_status silu_mat_set_shape(silu_mat A, int lanes, int passes, int chunk);
  * Time r = b - A x (one right-hand side) for each launch shape of the staged
  * kernel (lanes 1/2/4, rows per lane 1/2/4 with one lane, gather width 8/16,
  * the narrow configuration, and the automatic choice), keep the fastest (as silu_mat_set_shape), and
- * return it with its time per product.  Blocks.  Results change only by
+ * return it with its time per product (for the automatic choice, the shape of
+ * its tiles).  Blocks.  Results change only by
  * summation order across lanes.  Device context only; an empty matrix keeps
  * the automatic shape and reports 0 ms.  Any output pointer may be NULL.
  */
@@ -418,10 +420,14 @@ void silu_ilu_destroy(silu_ilu F);
 silu_status silu_ilu_set_lanes(silu_ilu F, int lanes_L, int lanes_U, int lanes_A);
 
 /*
- * Sweep kernel variant: 0 = automatic (the staged kernel for one right-hand
- * side; for 2 or 4 interleaved right-hand sides the staged kernel on
- * factors tiled one lane per row when the factor has at least 16 tiles per
- * multiprocessor, the lanes-per-row kernel otherwise), 1 = always the
+ * Sweep kernel variant: 0 = automatic (the sliced kernel, on a padded copy of
+ * the factor in slices of 32 rows, wherever padding adds at most two fifths
+ * to the entries: for one right-hand side with the bits of the staged kernel,
+ * for 2 to 4 interleaved ones of an FP64 smoother in column order; without
+ * such a copy the staged kernel for one right-hand side, and for 2 or 4 the
+ * staged kernel on factors tiled one lane per row when the factor has at
+ * least 16 tiles per multiprocessor, the lanes-per-row kernel otherwise),
+ * 1 = always the
  * lanes-per-row kernel, 2 = the staged kernel wherever it applies, 3 = as 2
  * but on length-sorted copies of the factors for one right-hand side (built
  * on first selection, for the factors where silu_ilu_layout shows sorting
@@ -611,7 +617,8 @@ silu_status silu_batch_fgmres(silu_batch B, double* x, const double* b, double t
  * candidate launch shape of the sweep kernels and keeps the fastest:
  * rows per warp (staged kernel: 8, 16, 32, 64 or 128 rows per warp tile,
  * i.e. four or two lanes per row, one, or one lane taking two or four rows;
- * or the lanes-per-row kernel with 2, 4 or 8 lanes) and gather width (8 or
+ * or the lanes-per-row kernel with 2, 4 or 8 lanes; or the library's default,
+ * variant 0) and gather width (8 or
  * 16 entries in flight per lane; 0 = the automatic configuration: narrow
  * tiles swept by 24 warps with 10 gathers in flight for FP64 factors whose
  * rows fit them, see silu_mat_set_shape, else 16).  Writes the chosen
@@ -621,8 +628,8 @@ silu_status silu_ilu_autotune(silu_ilu F, int sweeps_L, int sweeps_U, int* choic
 /*
  * The autotuner's candidates and their times from the last silu_ilu_autotune
  * on F: *count = number of candidates (0 before any tuning); for the first
- * min(cap, *count) candidates, shape[4 k .. 4 k + 3] = {variant (1 lanes-per-
- * row kernel, 2 staged kernel, 3 staged kernel on sorted copies), lanes per
+ * min(cap, *count) candidates, shape[4 k .. 4 k + 3] = {variant (0 the
+ * default, the sliced kernel where there is a copy, 1 lanes-per-row kernel, 2 staged kernel, 3 staged kernel on sorted copies), lanes per
  * row (0 = from the mean row length), rows per lane (0 = automatic), gather
  * width (0 = automatic)} and ms[k] = time per application (-1 for a candidate not run: a
  * sorted-copy candidate when no factor has one).  shape and ms may be NULL.

@@ -14,10 +14,10 @@ int auto_tile_nnz(const Csr& T, bool fp32, int lanes, int passes) {
 }
 
 // Uploads T (row pointers, columns, values in FP64 or FP32) as
-// 16-byte-rounded copies, and builds the row tiles of the staged kernel in
-// the automatic launch shape.
+// 16-byte-rounded copies, builds the row tiles of the staged kernel in the
+// automatic launch shape and the sliced copy where it pays (`copies`).
 cudaError_t upload_csr(const silu::Csr& T, bool fp32, DBuf& rp, DBuf& ci, DBuf& va, DBuf& tiles, DevCsr& d,
-                       cudaStream_t s) {
+                       cudaStream_t s, Copies copies) {
   const size_t n = (size_t)T.n, nnz = (size_t)T.nnz();
   const size_t vs = fp32 ? sizeof(float) : sizeof(double);
   std::vector<int32_t> rp32(T.rp.begin(), T.rp.end());
@@ -39,6 +39,16 @@ cudaError_t upload_csr(const silu::Csr& T, bool fp32, DBuf& rp, DBuf& ci, DBuf& 
       e = cudaMemcpyAsync(va.p, T.va.data(), sizeof(double) * nnz, cudaMemcpyHostToDevice, s);
     }
   }
+  d.n = (int)T.n;
+  d.nnz = T.nnz();
+  d.rp = rp.as<int>();
+  d.ci = ci.as<int>();
+  d.va = va.p;
+  d.fp32 = fp32;
+  d.explicit_shape = false;
+  d.sl.reset();
+  const bool slice = copies != Copies::kCsr && silu::slices_pay(T.rp.data(), T.n, fp32);
+  if (e == cudaSuccess && slice) e = silu::build_slices(T.rp.data(), d, s);
   std::vector<int> tl;
   const int tlanes = silu::staged_lanes(T.rp.data(), T.n);
   const int tpasses = silu::staged_passes(T.rp.data(), T.n, tlanes);
@@ -46,18 +56,42 @@ cudaError_t upload_csr(const silu::Csr& T, bool fp32, DBuf& rp, DBuf& ci, DBuf& 
   const bool tiled = silu::make_tiles(T.rp.data(), T.n, tlanes, tpasses, tl, tnnz);
   if (e == cudaSuccess && tiled) e = upload(tiles, tl.data(), tl.size(), s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // host staging vectors die at return
-  d.n = (int)T.n;
-  d.nnz = T.nnz();
-  d.rp = rp.as<int>();
-  d.ci = ci.as<int>();
-  d.va = va.p;
-  d.fp32 = fp32;
   d.tiles = tiled ? tiles.as<int4>() : nullptr;
   d.ntiles = tiled ? (int)(tl.size() / 4) : 0;
   d.tile_lanes = tlanes;
   d.tile_passes = tpasses;
   d.tile_nnz = tnnz;
+  if (e == cudaSuccess && d.sl && copies == Copies::kSmaller) {
+    if (tiled && d.sl->bytes > rp.bytes + ci.bytes + va.bytes + tiles.bytes) {
+      d.sl.reset();
+    } else {
+      for (DBuf* b : {&rp, &ci, &va, &tiles}) b->release();
+      d.rp = d.ci = nullptr;
+      d.va = nullptr;
+      d.tiles = nullptr;
+      d.ntiles = 0;
+    }
+  }
   return e;
+}
+
+// After a failed allocation of F's workspace: drop the sliced copies of F and
+// A, whose sweeps then run on the tiles (the same bits).  False if there was
+// nothing to drop.
+bool drop_slices(silu_ilu F) {
+  bool any = false;
+  for (DevCsr* d : {&F->A->d, &F->dL, &F->dU}) {
+    if (!d->sl || !d->rp) continue;
+    d->sl.reset();
+    any = true;
+  }
+  if (any) {
+    cudaGetLastError();
+    F->ws.drop_graphs();
+    F->config_gen++;
+    F->A->gen++;
+  }
+  return any;
 }
 
 cudaError_t upload_sorted(const Csr& T, bool fp32, SortedBufs& b, DevCsr& d, cudaStream_t s) {
@@ -85,7 +119,7 @@ cudaError_t upload_sorted(const Csr& T, bool fp32, SortedBufs& b, DevCsr& d, cud
   S.ci.swap(sci);
   S.va.swap(sva);
   DevCsr sd;
-  cudaError_t e = upload_csr(S, fp32, b.rp, b.ci, b.va, b.tiles, sd, s);
+  cudaError_t e = upload_csr(S, fp32, b.rp, b.ci, b.va, b.tiles, sd, s, Copies::kCsr);
   std::vector<int> tl;
   if (e == cudaSuccess && !silu::make_tiles(S.rp.data(), S.n, 1, 1, tl)) return cudaSuccess;
   if (e == cudaSuccess) e = upload(b.tiles, tl.data(), tl.size(), s);
@@ -110,6 +144,7 @@ namespace {
 // row and rl rows per lane, gather width.
 cudaError_t keep_shape(const Csr& h, DBuf& tiles, DevCsr& T, const DevCsr& old, cudaStream_t s) {
   T.chunk = old.chunk;
+  T.explicit_shape = old.explicit_shape;
   if (old.tile_lanes == T.tile_lanes && old.tile_passes == T.tile_passes && old.tile_nnz == T.tile_nnz)
     return cudaSuccess;
   // narrow tiles only where the new values' rows still fit them
@@ -152,8 +187,9 @@ cudaError_t upload_factors(silu_ilu F) {
   const DevCsr oldL = F->dL, oldU = F->dU;
   F->ws.drop_graphs();  // captured launches refer to the shapes and arrays replaced here
   F->config_gen++;
-  cudaError_t e = upload_csr(F->F.L, f32, F->L_rp, F->L_ci, F->L_va, F->L_tiles, F->dL, s);
-  if (e == cudaSuccess) e = upload_csr(Ut, f32, F->U_rp, F->U_ci, F->U_va, F->U_tiles, F->dU, s);
+  const Copies cp = F->ctx->factor_copies;
+  cudaError_t e = upload_csr(F->F.L, f32, F->L_rp, F->L_ci, F->L_va, F->L_tiles, F->dL, s, cp);
+  if (e == cudaSuccess) e = upload_csr(Ut, f32, F->U_rp, F->U_ci, F->U_va, F->U_tiles, F->dU, s, cp);
   if (e == cudaSuccess && F->sorted_ready) {  // sorted copies in use: rebuild them from the new values
     F->sorted_ready = false;
     e = ensure_sorted(F);
@@ -171,7 +207,9 @@ silu_status device_ok(silu_ctx ctx) {
   return SILU_OK;
 }
 
-cudaError_t ensure_vectors(silu_ilu F, int nrhs) {
+namespace {
+
+cudaError_t allocate_vectors(silu_ilu F, int nrhs) {
   const size_t bytes = sizeof(double) * (size_t)F->F.L.n * (size_t)nrhs;
   Workspace& w = F->ws;
   if (bytes <= w.vec_bytes && w.r.p) return cudaSuccess;
@@ -185,7 +223,7 @@ cudaError_t ensure_vectors(silu_ilu F, int nrhs) {
   return cudaSuccess;
 }
 
-cudaError_t ensure_krylov(silu_ilu F, int m) {
+cudaError_t allocate_krylov(silu_ilu F, int m) {
   Workspace& w = F->ws;
   if (m <= w.restart && w.V.p) return cudaSuccess;
   w.drop_graphs();
@@ -204,6 +242,19 @@ cudaError_t ensure_krylov(silu_ilu F, int m) {
   if ((e = w.scal.ensure(sizeof(double) * 8)) != cudaSuccess) return e;
   w.restart = m;
   return cudaSuccess;
+}
+
+}  // namespace
+
+// The workspace comes before the sliced copies where memory holds only one.
+cudaError_t ensure_vectors(silu_ilu F, int nrhs) {
+  const cudaError_t e = allocate_vectors(F, nrhs);
+  return e == cudaErrorMemoryAllocation && drop_slices(F) ? allocate_vectors(F, nrhs) : e;
+}
+
+cudaError_t ensure_krylov(silu_ilu F, int m) {
+  const cudaError_t e = allocate_krylov(F, m);
+  return e == cudaErrorMemoryAllocation && drop_slices(F) ? allocate_krylov(F, m) : e;
 }
 
 namespace {
@@ -392,13 +443,14 @@ cudaError_t ensure_direct(silu_ilu F) {
                           cudaMemcpyHostToDevice, s);
     F->dL64.va = F->L64_va.p;
     F->dL64.fp32 = false;
+    F->dL64.sl.reset();  // an FP32 copy
   }
   if (e != cudaSuccess) return e;
   // FP64 Utilde_s: reuse when the sweeps use it in FP64
   if (F->prec == SILU_FP64 && scaled_upper(F)) {
     F->dS64 = F->dU;
   } else {
-    e = upload_csr(F->Us, false, F->S_rp, F->S_ci, F->S_va, F->S_tiles, F->dS64, s);
+    e = upload_csr(F->Us, false, F->S_rp, F->S_ci, F->S_va, F->S_tiles, F->dS64, s, Copies::kCsr);
     if (e != cudaSuccess) return e;
   }
   e = upload(F->levLrows_d, F->levLrows.data(), F->levLrows.size(), s);
@@ -413,18 +465,38 @@ cudaError_t ensure_direct(silu_ilu F) {
 }
 
 
-// One sweep-shaped launch: the staged kernel for a single right-hand side
-// when the matrix has a tile partition (and the variant allows it), on the
-// length-sorted copy when that is selected, else the lanes-per-row kernel.
+// Whether several right-hand sides take the tiled multi-column sweep: it reads
+// each factor entry once for all R columns; on small systems (fewer tiles
+// than a grid of warps has) its pipeline start costs more than it saves,
+// unless a staged variant was asked for explicitly.
+bool multi_tiles(silu_ilu F, const DevCsr& T, int R) {
+  return F->variant != 1 && silu::staged_multi_ok(T, R) && (F->variant >= 2 || T.ntiles >= F->ctx->env.sms * 16);
+}
+
+// Whether a launch on T takes the sliced copy: the default wherever there is
+// one.  An explicit staged shape of A (silu_mat_set_shape) and, for the
+// factors, an explicit staged variant (2, 3) keep the tiles; variant 1 keeps
+// the lanes-per-row kernel everywhere.
+bool use_slices(silu_ilu F, const DevCsr& T, int R, int ldx) {
+  if (!T.sl || T.explicit_shape || F->variant == 1 || R > 4 || (R == 1 && ldx != 1)) return false;
+  if (F->variant != 0 && (&T == &F->dL || &T == &F->dU)) return false;
+  // several columns of an FP32 smoother: only where the tiled multi-column
+  // sweep, which sums in the same order, would run (an FP32 sum in another
+  // order differs by 1e-7)
+  if (R > 1 && F->prec == SILU_FP32) return multi_tiles(F, T, R);
+  return true;
+}
+
+// One sweep-shaped launch: the sliced kernel by default; else the staged
+// kernel for a single right-hand side when the matrix has a tile partition
+// (and the variant allows it), on the length-sorted copy when that is
+// selected; else the lanes-per-row kernel.
 cudaError_t sweep_launch(silu_ilu F, const DevCsr& T, silu::Mode mode, int R, int lanes, int ldx, const void* c,
                          const void* in, void* out, const double* dinv, double* x, int epi) {
   cudaStream_t s = F->ctx->stream;
-  // several right-hand sides: the staged kernel reads each factor entry once
-  // for all R columns; on small systems (fewer tiles than a grid of warps
-  // has) its pipeline start costs more than it saves, unless a staged
-  // variant was asked for explicitly
-  if (R > 1 && F->variant != 1 && silu::staged_multi_ok(T, R) &&
-      (F->variant >= 2 || T.ntiles >= F->ctx->env.sms * 16))
+  if (use_slices(F, T, R, ldx))
+    return silu::launch_sweep_slices(T, mode, F->ctx->env, R, ldx, c, in, out, dinv, x, epi, s);
+  if (R > 1 && multi_tiles(F, T, R))
     return silu::launch_sweep_staged_multi(T, mode, F->ctx->env, R, ldx, c, in, out, dinv, x, epi, s);
   if (R == 1 && ldx == 1 && T.ntiles > 0 && F->variant != 1) {
     if (F->variant != 3 || T.nstiles == 0) return silu::launch_sweep_staged(T, mode, F->ctx->env, c, in, out, dinv, x, epi, s);
@@ -762,6 +834,18 @@ void direct_chunk(silu_ilu F, double* x, const double* b, int R, int ldx, size_t
 
 int chunk_width(int left) { return left >= 4 ? 4 : (left >= 2 ? 2 : 1); }
 
+// Column blocks of the sliced kernel: up to four columns, three where that
+// leaves no single column behind (a factor is read once per block).
+int slice_width(int left) { return left == 5 || left == 3 ? 3 : chunk_width(left); }
+
+// Columns of the next block of a smoother application with `left` to go.
+int smooth_width(silu_ilu F, int left, int ldx) {
+  const DevCsr* T[3] = {&F->A->d, &F->dL, &F->dU};
+  for (const DevCsr* t : T)
+    if (!use_slices(F, *t, 3, ldx)) return chunk_width(left);
+  return F->fused_mode == 2 ? chunk_width(left) : slice_width(left);
+}
+
 
 namespace {
 
@@ -931,6 +1015,7 @@ silu_status silu_ctx_create(int device, void* cuda_stream, silu_ctx* out) {
     if (e == cudaSuccess) e = cudaMalloc((void**)&c->env.err, 4 * sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(c->env.err, 0, 4 * sizeof(int));
     if (e == cudaSuccess) e = silu::staged_prepare();
+    if (e == cudaSuccess) e = silu::slices_prepare();
     if (e != cudaSuccess) {
       delete c;
       return SILU_ERR_CUDA;
@@ -1043,7 +1128,8 @@ int candidate_tile_nnz(const Csr& h, bool fp32, int g, int rl, int chunk) {
 // length) and `passes` rows per lane (0 = automatic), gather width `chunk`;
 // variant 3: staged kernel on the length-sorted copies (where they exist;
 // one lane per row), gather width `chunk`;
-// variant 1: lanes-per-row kernel with `lanes` lanes.
+// variant 1: lanes-per-row kernel with `lanes` lanes;
+// variant 0: the library's default (the sliced kernel where there is a copy).
 struct TuneCandidate {
   int variant, lanes, passes, chunk;
 };
@@ -1053,7 +1139,8 @@ struct TuneCandidate {
 // configuration where it fits.
 const TuneCandidate kTune[] = {{2, 0, 0, 0},  {2, 0, 0, 16}, {2, 0, 0, 8},  {2, 1, 1, 16}, {2, 1, 2, 16},
                                {2, 1, 4, 16}, {2, 1, 4, 8},  {2, 2, 1, 16}, {2, 4, 1, 16}, {1, 2, 0, 16},
-                               {1, 4, 0, 16}, {1, 8, 0, 16}, {3, 1, 1, 16}, {3, 1, 1, 8}};
+                               {1, 4, 0, 16}, {1, 8, 0, 16}, {3, 1, 1, 16}, {3, 1, 1, 8},
+                               {0, 0, 0, 0}};
 
 }  // namespace
 
@@ -1240,7 +1327,7 @@ silu_status silu_mat_create(silu_ctx ctx, int64_t n, int64_t nnz, const int64_t*
         delete M;
         return ds;
       }
-      cudaError_t e = upload_csr(M->A, false, M->rp, M->ci, M->va, M->tiles, M->d, ctx->stream);
+      cudaError_t e = upload_csr(M->A, false, M->rp, M->ci, M->va, M->tiles, M->d, ctx->stream, ctx->copies);
       if (e != cudaSuccess) {
         delete M;
         return cuda_err(ctx, e, "upload of A");
@@ -1288,6 +1375,7 @@ silu_status silu_mat_set_shape(silu_mat A, int lanes, int passes, int chunk) {
   A->d.tile_passes = rl;
   A->d.tile_nnz = lim;
   A->d.chunk = (chunk == 8) ? 8 : 16;
+  A->d.explicit_shape = lanes != 0 || passes != 0 || chunk != 0;  // (0, 0, 0): the sliced copy where there is one
   A->gen++;
   return SILU_OK;
 }
@@ -1365,7 +1453,14 @@ silu_status silu_mat_residual(silu_mat A, double* r, const double* x, const doub
   if (A->A.n == 0) return SILU_OK;
   cudaStream_t s = ctx->stream;
   try {
-    if (nrhs == 1 && A->d.ntiles > 0) {
+    if (A->d.sl && !A->d.explicit_shape) {
+      for (int c0 = 0; c0 < nrhs;) {
+        const int w = slice_width(nrhs - c0);
+        LAUNCH(ctx, SILU_K_RESIDUAL, silu::launch_sweep_slices(A->d, silu::MODE_D, ctx->env, w, nrhs, b + c0, x + c0,
+                                                               r + c0, nullptr, nullptr, silu::EPI_STORE, s));
+        c0 += w;
+      }
+    } else if (nrhs == 1 && A->d.ntiles > 0) {
       LAUNCH(ctx, SILU_K_RESIDUAL, silu::launch_sweep_staged(A->d, silu::MODE_D, ctx->env, b, x, r, nullptr, nullptr,
                                                              silu::EPI_STORE, s));
     } else {
@@ -1543,6 +1638,7 @@ silu_status ilu_refactor(silu_ilu F, const double* new_val) {
       if (ds != SILU_OK) return ds;
       cudaStream_t s = ctx->stream;
       cudaError_t e = upload(F->A->va, A.va.data(), A.va.size(), s);
+      if (e == cudaSuccess) e = silu::refill_slices(F->A->d, s);
       if (e == cudaSuccess) e = upload_factors(F);
       if (e == cudaSuccess) e = upload(F->d_dinv, F->dinv.data(), F->dinv.size(), s);
       if (e == cudaSuccess && !F->dcol.empty()) e = upload(F->d_dcol, F->dcol.data(), F->dcol.size(), s);
@@ -1579,7 +1675,7 @@ silu_status ilu_smooth(silu_ilu F, double* x, const double* b, int nrhs, int swe
   try {
     CK(ensure_vectors(F, nrhs));
     for (int c0 = 0; c0 < nrhs;) {
-      const int R = chunk_width(nrhs - c0);
+      const int R = smooth_width(F, nrhs - c0, nrhs);
       smooth_chunk(F, x + c0, b + c0, R, nrhs, (size_t)c0, sweeps_L, sweeps_U, false);
       c0 += R;
     }

@@ -324,7 +324,7 @@ int grid_for(silu_batch B) {
   return want < cap ? (want > 0 ? want : 1) : cap;
 }
 
-cudaError_t ensure_bkrylov(silu_batch B, int m) {
+cudaError_t allocate_bkrylov(silu_batch B, int m) {
   if (B->restart >= m && B->V.p) return cudaSuccess;
   for (InnerGraph& ig : B->graphs)
     if (ig.exec) cudaGraphExecDestroy(ig.exec);
@@ -351,6 +351,11 @@ cudaError_t ensure_bkrylov(silu_batch B, int m) {
   if ((e = B->counter.ensure(sizeof(int) * 4)) != cudaSuccess) return e;
   B->restart = m;
   return cudaSuccess;
+}
+
+cudaError_t ensure_bkrylov(silu_batch B, int m) {
+  const cudaError_t e = allocate_bkrylov(B, m);
+  return e == cudaErrorMemoryAllocation && drop_slices(B->F) ? allocate_bkrylov(B, m) : e;
 }
 
 // The fixed kernel sequence of inner iteration j (on the batch's buffers).

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -50,6 +51,30 @@ constexpr int kTileNnzNarrow = 360;
 constexpr int kNarrowChunkRows = 10;
 constexpr double kNarrowMeanRow = 9.0;
 
+// A matrix cut into slices of 32 consecutive rows, for k_slices (one warp per
+// slice, one lane per row; kernels_slices.cu).  Slice s holds, for k < width
+// (its longest row), entry k of every row, padded with value 0 and an
+// all-ones column; the entries of rows k and k + 1 of a lane are adjacent
+// ([k / 2][lane][2], a last odd row as [lane]), so a lane reads two entries
+// at once.  Columns are 16-bit offsets from the slice's smallest column where
+// every slice's columns span less than 65535, else int32.
+struct Slices {
+  int ns = 0;
+  int64_t slots = 0;      // stored entries, padding included
+  int widest = 0;         // entries of the longest row
+  int lanes = 1;          // partial sums per row: the lanes the tiled sweep gives it (staged_lanes)
+  bool wide = false;      // int32 columns instead of 16-bit offsets
+  int2* hdr = nullptr;    // ns + 1 entries: {first slot, smallest column}
+  void* ci = nullptr;     // uint16_t offsets, or int columns
+  void* va = nullptr;     // double or float
+  void* buf = nullptr;    // the one allocation that holds the three
+  size_t bytes = 0;       // and its size
+  Slices() = default;
+  Slices(const Slices&) = delete;
+  Slices& operator=(const Slices&) = delete;
+  ~Slices();
+};
+
 struct DevCsr {
   int n = 0;
   int64_t nnz = 0;
@@ -79,6 +104,10 @@ struct DevCsr {
   int tile_passes = 1; // rows per lane in a tile (1, 2 or 4; only with one lane per row)
   int chunk = 16;      // entries gathered per lane before the FMAs (8 or 16)
   int tile_nnz = kTileNnz;  // the entry limit the tiles were cut with (kTileNnzNarrow: narrow configuration)
+  // the sliced copy (null: none); swept instead of the tiles unless a staged
+  // launch shape was asked for (explicit_shape) or a sweep variant says so
+  std::shared_ptr<Slices> sl;
+  bool explicit_shape = false;
 };
 
 
@@ -179,6 +208,33 @@ bool staged_multi_ok(const DevCsr& T, int R);
 cudaError_t launch_sweep_staged_multi(const DevCsr& T, Mode mode, const LaunchEnv& env, int R, int ldx, const void* c,
                                       const void* in, void* out, const double* dinv, double* x, int epi,
                                       cudaStream_t s);
+// The sweep on the sliced copy T.sl for R = 1..4 interleaved right-hand sides
+// (leading dimension ldx >= R); with one column the bits of the tiled sweep
+// in its automatic shape.
+cudaError_t launch_sweep_slices(const DevCsr& T, Mode mode, const LaunchEnv& env, int R, int ldx, const void* c,
+                                const void* in, void* out, const double* dinv, double* x, int epi, cudaStream_t s);
+// Whether a matrix with this row pointer gets a sliced copy (see the
+// definition for the limit on padding).
+bool slices_pay(const int64_t* rp, int64_t n, bool fp32);
+// Build d.sl on the device from d's uploaded CSR arrays (rp: the host row
+// pointer, for which slices_pay holds).  A failed allocation leaves d.sl null
+// and is not an error.  Blocks on s until the headers are copied.
+cudaError_t build_slices(const int64_t* rp, DevCsr& d, cudaStream_t s);
+// New values on the same pattern: fill d.sl again from d's CSR arrays (on s).
+cudaError_t refill_slices(const DevCsr& d, cudaStream_t s);
+// Give the slice kernels' instantiations the whole L1 (once per context).
+cudaError_t slices_prepare();
+// The part of both for several right-hand sides (a translation unit of its own).
+cudaError_t slices_prepare_multi();
+// The FP32 sweep of large matrices for one right-hand side, its matrix stream
+// staged through shared memory (kernels_slices_ring.cu).
+cudaError_t slices_prepare_ring();
+bool slices_ring_fits(const DevCsr& T, Mode mode, int sms);
+cudaError_t launch_slices_ring(const DevCsr& T, const LaunchEnv& env, const void* c, const void* in, void* out,
+                               const double* dinv, double* x, int epi, cudaStream_t s);
+cudaError_t launch_slices_multi(const DevCsr& T, Mode mode, const LaunchEnv& env, int R, int ldx, const void* c,
+                                const void* in, void* out, const double* dinv, double* x, int epi, cudaStream_t s);
+
 // Opt every staged-kernel instantiation into its shared-memory size on the
 // current device (done once per context, before any stream capture).
 cudaError_t staged_prepare();

@@ -60,8 +60,15 @@ struct DBuf {
 using silu::DBuf;
 using silu::DevCsr;
 
+// Device copies of an uploaded matrix: CSR arrays with tiles, those and the
+// sliced copy where it pays, or the smaller of the two (the solve server, whose
+// memory estimate counts one copy; calls that read the CSR arrays then fail).
+enum class Copies { kCsr, kBoth, kSmaller };
+
 struct silu_ctx_s {
   int device = -1;
+  Copies copies = Copies::kBoth;         // of matrices and hierarchy operators
+  Copies factor_copies = Copies::kBoth;  // of sweep factors
   cudaStream_t stream = nullptr;
   std::string err;
   double* pinned = nullptr;  // small host buffer for scalar read-backs
@@ -354,7 +361,9 @@ cudaError_t upload(DBuf& b, const T* src, size_t count, cudaStream_t s) {
 // float.  Arrays get kCsrPad spare (zeroed) elements for the staged kernel's
 
 cudaError_t upload_csr(const Csr& T, bool fp32, DBuf& rp, DBuf& ci, DBuf& va, DBuf& tiles, DevCsr& d,
-                       cudaStream_t s);
+                       cudaStream_t s, Copies copies = Copies::kBoth);
+// Drop the sliced copies of F's factors and of A (false if there are none).
+bool drop_slices(silu_ilu F);
 // The tile entry limit of the automatic launch shape: narrow tiles for FP64
 // values with one lane per row whose rows fit them (silu::narrow_fits).
 int auto_tile_nnz(const Csr& T, bool fp32, int lanes, int passes);

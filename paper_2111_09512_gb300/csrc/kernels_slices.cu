@@ -1,0 +1,251 @@
+// Building the sliced copy of a matrix on the device, and the sliced sweep
+// for one right-hand side (see slices.cuh).
+#include "slices.cuh"
+
+#include <algorithm>
+#include <new>
+#include <vector>
+
+namespace silu {
+
+Slices::~Slices() {
+  if (buf) cudaFree(buf);
+}
+
+namespace {
+
+// A sliced copy is made where padding adds at most two fifths to the entries
+// (and for any matrix of a few slices).  Padding costs FP64 sweeps issue time
+// and every sweep bytes: the 128^3 cut-cell ILUT lower factor (1.26 slots per
+// entry) takes 44.0 us sliced against 45.9 us tiled; of the AMG operators of
+// the 128^3 cut-cell matrix, those within 1.4 gain (V-cycle 743 -> 732 us
+// against a limit of 1.2) and taking those up to 1.7 as well, rows of 30 and
+// more entries of uneven length, loses (843 us).
+constexpr double kSlicePadMax = 1.4;
+constexpr double kSlicePadFree = 2048.0;
+constexpr int64_t kMaxSlots = (int64_t)INT32_MAX - 65536;  // slot numbers (and a chunk beyond the last) fit an int
+
+// The slots of all slices (their first slots into *hdr, the longest row of all into *widest).
+int64_t slice_widths(const int64_t* rp, int64_t n, std::vector<int2>* hdr, int* widest = nullptr) {
+  int64_t slots = 0, most = 0;
+  const int64_t ns = (n + 31) / 32;
+  if (hdr) hdr->resize((size_t)ns + 1);
+  for (int64_t s = 0; s < ns; ++s) {
+    if (hdr) (*hdr)[(size_t)s] = make_int2((int)slots, 0);
+    int64_t w = 0;
+    for (int64_t r = s * 32; r < std::min<int64_t>(n, s * 32 + 32); ++r) w = std::max<int64_t>(w, rp[r + 1] - rp[r]);
+    slots += 32 * w;
+    most = std::max(most, w);
+    if (slots > kMaxSlots) return slots;
+  }
+  if (hdr) (*hdr)[(size_t)ns] = make_int2((int)slots, 0);
+  if (widest) *widest = (int)most;
+  return slots;
+}
+
+// Smallest column of every slice into its header, largest span of any slice
+// into *span (at least 0).  One warp per slice.
+__global__ void k_slice_span(int ns, int n, const int* __restrict__ rp, const int* __restrict__ ci,
+                             int2* __restrict__ hdr, int* __restrict__ span) {
+  const int s = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5);
+  const int lane = threadIdx.x & 31;
+  if (s >= ns) return;
+  const int r0 = s * 32, r1 = min(n, r0 + 32);
+  int lo = INT32_MAX, hi = -1;
+  for (int p = rp[r0] + lane; p < rp[r1]; p += 32) {
+    lo = min(lo, ci[p]);
+    hi = max(hi, ci[p]);
+  }
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  if (lane == 0) {
+    hdr[s].y = hi < 0 ? 0 : lo;
+    if (hi >= 0) atomicMax(span, hi - lo);
+  }
+}
+
+// Fill the slices from the CSR arrays: one warp per slice, one lane per row.
+template <class MT, class CT>
+__global__ void k_slice_fill(int ns, int n, const int* __restrict__ rp, const int* __restrict__ ci,
+                             const MT* __restrict__ va, const int2* __restrict__ hdr, CT* __restrict__ sci,
+                             MT* __restrict__ sva) {
+  const int s = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5);
+  const int lane = threadIdx.x & 31;
+  if (s >= ns) return;
+  const int2 h = hdr[s];
+  const int width = (hdr[s + 1].x - h.x) >> 5;
+  const int r = s * 32 + lane;
+  const int b = r < n ? rp[r] : 0;
+  const int len = r < n ? rp[r + 1] - b : 0;
+  for (int k = 0; k < width; ++k) {
+    const int at = (k | 1) < width ? h.x + 64 * (k >> 1) + 2 * lane + (k & 1) : h.x + 32 * k + lane;
+    CT c = (CT)~(CT)0;
+    MT v = MT(0);
+    if (k < len) {
+      c = (CT)(sizeof(CT) == 2 ? ci[b + k] - h.y : ci[b + k]);
+      v = va[b + k];
+    }
+    sci[at] = c;
+    sva[at] = v;
+  }
+}
+
+template <class MT>
+cudaError_t fill(const DevCsr& d, const Slices& S, cudaStream_t s) {
+  const unsigned blocks = (unsigned)((S.ns + 7) / 8);
+  if (S.wide)
+    k_slice_fill<MT, int><<<blocks, 256, 0, s>>>(S.ns, d.n, d.rp, d.ci, (const MT*)d.va, S.hdr, (int*)S.ci,
+                                                 (MT*)S.va);
+  else
+    k_slice_fill<MT, uint16_t><<<blocks, 256, 0, s>>>(S.ns, d.n, d.rp, d.ci, (const MT*)d.va, S.hdr, (uint16_t*)S.ci,
+                                                      (MT*)S.va);
+  return cudaGetLastError();
+}
+
+// FP64 for one right-hand side: one pair per chunk and 48 warps per SM (128^3
+// ILUT application 820 us; two pairs and 32 or 40 warps 896 / 893, three and
+// 32 830; 160^3 27-point residual 232 us against 236 / 227 / 240), which no
+// register spills; four partial sums need a chunk of four entries.
+template <class VO, class CT, int LN>
+using Double1 = SliceKernel<double, double, VO, CT, 1, LN == 4 ? 2 : 1, LN == 4 ? 4 : 6, false, LN>;
+
+template <class VO, class CT>
+cudaError_t double1(const DevCsr& T, const LaunchEnv& env, const void* c, const void* in, void* out,
+                    const double* dinv, double* x, int epi, cudaStream_t s) {
+  switch (T.sl->lanes) {
+    case 1: return Double1<VO, CT, 1>::launch(T, env, 1, c, in, out, dinv, x, epi, s);
+    case 2: return Double1<VO, CT, 2>::launch(T, env, 1, c, in, out, dinv, x, epi, s);
+    case 4: return Double1<VO, CT, 4>::launch(T, env, 1, c, in, out, dinv, x, epi, s);
+  }
+  return cudaErrorInvalidValue;
+}
+
+// Every instance that launch_sweep_slices picks for one right-hand side.
+template <class F>
+cudaError_t for_each_shape(F f) {
+  cudaError_t e = cudaSuccess;
+  auto add = [&](cudaError_t r) {
+    if (e == cudaSuccess) e = r;
+  };
+  add(f(Double1<double, uint16_t, 1>()));
+  add(f(Double1<double, uint16_t, 2>()));
+  add(f(Double1<double, uint16_t, 4>()));
+  add(f(Double1<double, int, 1>()));
+  add(f(Double1<double, int, 2>()));
+  add(f(Double1<double, int, 4>()));
+  add(f(Double1<float, uint16_t, 1>()));
+  add(f(Double1<float, uint16_t, 2>()));
+  add(f(Double1<float, uint16_t, 4>()));
+  add(f(Double1<float, int, 1>()));
+  add(f(Double1<float, int, 2>()));
+  add(f(Double1<float, int, 4>()));
+  add(f(SliceKernel<float, float, float, uint16_t, 1, 2, 6, false>()));
+  add(f(SliceKernel<float, float, float, uint16_t, 1, 4, 3, false>()));
+  add(f(SliceKernel<float, float, float, uint16_t, 1, 7, 3, false>()));
+  add(f(SliceKernel<float, float, float, int, 1, 2, 5, false>()));
+  add(f(SliceKernel<float, float, float, int, 1, 4, 3, false>()));
+  return e;
+}
+
+}  // namespace
+
+bool slices_pay(const int64_t* rp, int64_t n, bool fp32) {
+  // FP32 rows of more than 16 entries on average keep the tiled sweep, whose
+  // lanes share a row (an FP32 sum in another order differs by 1e-7)
+  if (n <= 0 || (fp32 && staged_lanes(rp, n) > 1)) return false;
+  const int64_t slots = slice_widths(rp, n, nullptr);
+  return slots <= kMaxSlots && (double)slots <= kSlicePadMax * (double)rp[n] + kSlicePadFree;
+}
+
+cudaError_t build_slices(const int64_t* rp, DevCsr& d, cudaStream_t s) {
+  d.sl.reset();
+  std::shared_ptr<Slices> S(new (std::nothrow) Slices);
+  if (!S) return cudaSuccess;
+  std::vector<int2> hdr;
+  S->slots = slice_widths(rp, d.n, &hdr, &S->widest);
+  S->ns = (int)hdr.size() - 1;
+  S->lanes = staged_lanes(rp, d.n);
+  // one allocation: the headers and, past them, one int for the span; values; columns
+  const size_t hb = (sizeof(int2) * (hdr.size() + 1) + 255) / 256 * 256;
+  const size_t slots = (size_t)std::max<int64_t>(S->slots, 32);
+  const size_t vb = ((d.fp32 ? sizeof(float) : sizeof(double)) * slots + 255) / 256 * 256;
+  auto allocate = [&](size_t col_bytes) {
+    S->bytes = hb + vb + col_bytes * slots;
+    const cudaError_t e = cudaMalloc(&S->buf, S->bytes);
+    S->hdr = (int2*)S->buf;
+    S->va = (char*)S->buf + hb;
+    S->ci = (char*)S->buf + hb + vb;
+    return e;
+  };
+  auto give_up = [](cudaError_t e) {
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();  // no room for the copy: the sweeps run on the CSR tiles
+    return cudaSuccess;
+  };
+  cudaError_t e = allocate(sizeof(uint16_t));
+  if (e != cudaSuccess) return give_up(e);
+  const unsigned blocks = (unsigned)((S->ns + 7) / 8);
+  for (;;) {
+    int* span = (int*)(S->hdr + hdr.size());
+    e = cudaMemcpyAsync(S->hdr, hdr.data(), sizeof(int2) * hdr.size(), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(span, 0, sizeof(int), s);
+    if (e != cudaSuccess) return e;
+    k_slice_span<<<blocks, 256, 0, s>>>(S->ns, d.n, d.rp, d.ci, S->hdr, span);
+    e = cudaGetLastError();
+    int widest = 0;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&widest, span, sizeof(int), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // hdr is a host vector of this call
+    if (e != cudaSuccess) return e;
+    if (widest < 65535 || S->wide) break;  // offset 65535 marks padding
+    S->wide = true;
+    cudaFree(S->buf);
+    S->buf = nullptr;
+    e = allocate(sizeof(int));
+    if (e != cudaSuccess) return give_up(e);
+  }
+  e = d.fp32 ? fill<float>(d, *S, s) : fill<double>(d, *S, s);
+  if (e == cudaSuccess) d.sl = std::move(S);
+  return e;
+}
+
+cudaError_t refill_slices(const DevCsr& d, cudaStream_t s) {
+  if (!d.sl) return cudaSuccess;
+  return d.fp32 ? fill<float>(d, *d.sl, s) : fill<double>(d, *d.sl, s);
+}
+
+cudaError_t slices_prepare() {
+  cudaError_t e = for_each_shape([](auto k) { return decltype(k)::prepare(); });
+  if (e == cudaSuccess) e = slices_prepare_ring();
+  return e == cudaSuccess ? slices_prepare_multi() : e;
+}
+
+cudaError_t launch_sweep_slices(const DevCsr& T, Mode mode, const LaunchEnv& env, int R, int ldx, const void* c,
+                                const void* in, void* out, const double* dinv, double* x, int epi, cudaStream_t s) {
+  if (!T.sl || R < 1 || R > 4 || ldx < R || (R == 1 && ldx != 1)) return cudaErrorInvalidValue;
+  if (R > 1) return launch_slices_multi(T, mode, env, R, ldx, c, in, out, dinv, x, epi, s);
+  if (slices_ring_fits(T, mode, env.sms)) return launch_slices_ring(T, env, c, in, out, dinv, x, epi, s);
+  const bool wide = T.sl->wide;
+  // FP32, which only small matrices reach: a whole row per chunk where rows
+  // allow (27-point 32^3 4.5 us a sweep).
+  const double mean = (double)T.sl->slots / (32.0 * (double)T.sl->ns);
+  auto go = [&](auto k) { return decltype(k)::launch(T, env, ldx, c, in, out, dinv, x, epi, s); };
+  switch (mode) {
+    case MODE_D:
+      return wide ? double1<double, int>(T, env, c, in, out, dinv, x, epi, s)
+                  : double1<double, uint16_t>(T, env, c, in, out, dinv, x, epi, s);
+    case MODE_DF:
+      return wide ? double1<float, int>(T, env, c, in, out, dinv, x, epi, s)
+                  : double1<float, uint16_t>(T, env, c, in, out, dinv, x, epi, s);
+    case MODE_F:
+      if (mean <= 4.0)
+        return wide ? go(SliceKernel<float, float, float, int, 1, 2, 5, false>())
+                    : go(SliceKernel<float, float, float, uint16_t, 1, 2, 6, false>());
+      if (wide || mean <= 8.0 || mean > 14.0)
+        return wide ? go(SliceKernel<float, float, float, int, 1, 4, 3, false>())
+                    : go(SliceKernel<float, float, float, uint16_t, 1, 4, 3, false>());
+      return go(SliceKernel<float, float, float, uint16_t, 1, 7, 3, false>());
+  }
+  return cudaErrorInvalidValue;
+}
+
+}  // namespace silu

@@ -30,7 +30,9 @@
 #include <cstdint>
 #include <vector>
 
+#include "bulk.cuh"
 #include "device.cuh"
+#include "sweep_ptx.cuh"
 
 namespace silu {
 
@@ -130,95 +132,6 @@ template <class MT>
 __host__ __device__ constexpr int warps_of() {
   return sizeof(MT) == 4 ? kWarpsF32 : kWarpsF64;
 }
-constexpr unsigned long long kWaitNs = 2000000000ull;  // 2 s bound on any wait
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void fence_mbar_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
-
-__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n"
-      " .reg .pred p;\n"
-      " mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-      " selp.u32 %0, 1, 0, p;\n"
-      "}\n"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
-// Wait for phase `parity` of bar, giving up after kWaitNs.  Returns false on timeout.
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const unsigned long long t0 = global_ns();
-  while (!mbar_try_wait(bar, parity))
-    if (global_ns() - t0 > kWaitNs) return false;
-  return true;
-}
-
-__device__ __forceinline__ uint64_t policy_evict_first() {
-  uint64_t p;
-  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
-  return p;
-}
-
-__device__ __forceinline__ uint64_t policy_evict_normal() {
-  uint64_t p;
-  asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
-  return p;
-}
-
-__device__ __forceinline__ uint64_t policy_evict_last() {
-  uint64_t p;
-  asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
-  return p;
-}
-
-// Vector accesses that keep the iterates resident in L2 across sweeps.
-__device__ __forceinline__ double ld_keep(const double* p, uint64_t pol) {
-  double v;
-  asm("ld.global.nc.L2::cache_hint.f64 %0, [%1], %2;" : "=d"(v) : "l"(p), "l"(pol));
-  return v;
-}
-__device__ __forceinline__ float ld_keep(const float* p, uint64_t pol) {
-  float v;
-  asm("ld.global.nc.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(p), "l"(pol));
-  return v;
-}
-__device__ __forceinline__ void st_keep(double* p, double v, uint64_t pol) {
-  asm volatile("st.global.L2::cache_hint.f64 [%0], %1, %2;" ::"l"(p), "d"(v), "l"(pol) : "memory");
-}
-__device__ __forceinline__ void st_keep(float* p, float v, uint64_t pol) {
-  asm volatile("st.global.L2::cache_hint.f32 [%0], %1, %2;" ::"l"(p), "f"(v), "l"(pol) : "memory");
-}
-
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar, uint64_t pol) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::"r"(
-          smem_u32(dst)),
-      "l"(src), "r"(bytes), "r"(smem_u32(bar)), "l"(pol)
-      : "memory");
-}
-
 // One stage: a 16-byte header (the tile descriptor, written by the issuing
 // lane), then values, column indices and row pointers as copied, and, for a
 // length-sorted layout, the tile's row numbers in the vectors.
@@ -258,80 +171,6 @@ __device__ __forceinline__ void issue_tile(int4 d, unsigned char* st, uint64_t* 
   if (bc) bulk_g2s(st + L::kHdr + L::kVal, ci + c0, bc, bar, pol);
   if (RP) bulk_g2s(st + L::kHdr + L::kVal + L::kCol, rp + q0, br, bar, pol);
   if (PERM && bp) bulk_g2s(st + L::kHdr + L::kVal + L::kCol + L::kRp, perm + q0, bp, bar, pol);
-}
-
-// Epilogue operands (dinv_row, x_row) are read after the accumulation; a
-// prefetch into L1 issued before it takes their memory latency off the end
-// of the tile without holding registers through the gathers.
-__device__ __forceinline__ void prefetch_l1(const void* p) {
-  asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
-}
-__device__ __forceinline__ void prefetch_epilogue(int epi, int row, const double* dinv, const double* x) {
-  switch (epi) {
-    case EPI_SCALE:
-      prefetch_l1(dinv + row);
-      break;
-    case EPI_SCALE_ADDX:
-    case EPI_JAC_ADDX:
-      prefetch_l1(dinv + row);
-      prefetch_l1(x + row);
-      break;
-    case EPI_SCALE_SETX:
-    case EPI_JAC:
-    case EPI_JAC_SETX:
-      prefetch_l1(dinv + row);
-      break;
-    case EPI_ADDX:
-    case EPI_RICH_ADDX:
-      prefetch_l1(x + row);
-      break;
-    default:
-      break;
-  }
-}
-
-// t = c_row - (T in)_row, already formed by the accumulation
-template <class MT, class VI, class VO>
-__device__ __forceinline__ void epilogue(int epi, int row, MT t, const VI* in, VO* out, const double* dinv,
-                                         double* x, uint64_t keep) {
-  switch (epi) {
-    case EPI_STORE: st_keep(out + row, (VO)t, keep); break;
-    case EPI_SCALE: st_keep(out + row, (VO)(dinv[row] * (double)t), keep); break;
-    case EPI_ADDX: x[row] += (double)t; break;
-    case EPI_SETX: x[row] = (double)t; break;
-    case EPI_SCALE_ADDX: x[row] += dinv[row] * (double)t; break;
-    case EPI_SCALE_SETX: x[row] = dinv[row] * (double)t; break;
-    case EPI_JAC: st_keep(out + row, (VO)((MT)in[row] + (MT)dinv[row] * t), keep); break;
-    case EPI_JAC_ADDX: x[row] += (double)((MT)in[row] + (MT)dinv[row] * t); break;
-    case EPI_JAC_SETX: x[row] = (double)((MT)in[row] + (MT)dinv[row] * t); break;
-    case EPI_RICH: st_keep(out + row, (VO)(t + (MT)in[row]), keep); break;
-    case EPI_RICH_ADDX: x[row] += (double)(t + (MT)in[row]); break;
-    case EPI_RICH_SETX: x[row] = (double)(t + (MT)in[row]); break;
-    default: break;
-  }
-}
-
-// The same epilogues for column k of R interleaved right-hand sides: vector
-// entries at o = row * ldx + k, dinv at row.
-template <class MT, class VI, class VO>
-__device__ __forceinline__ void epilogue_col(int epi, int row, size_t o, MT t, const VI* in, VO* out,
-                                             const double* dinv, double* x, uint64_t keep) {
-  switch (epi) {
-    case EPI_STORE: st_keep(out + o, (VO)t, keep); break;
-    case EPI_SCALE: st_keep(out + o, (VO)(dinv[row] * (double)t), keep); break;
-    case EPI_ADDX: x[o] += (double)t; break;
-    case EPI_SETX: x[o] = (double)t; break;
-    case EPI_SCALE_ADDX: x[o] += dinv[row] * (double)t; break;
-    case EPI_SCALE_SETX: x[o] = dinv[row] * (double)t; break;
-    case EPI_JAC: st_keep(out + o, (VO)((MT)in[o] + (MT)dinv[row] * t), keep); break;
-    case EPI_JAC_ADDX: x[o] += (double)((MT)in[o] + (MT)dinv[row] * t); break;
-    case EPI_JAC_SETX: x[o] = (double)((MT)in[o] + (MT)dinv[row] * t); break;
-    case EPI_RICH: st_keep(out + o, (VO)(t + (MT)in[o]), keep); break;
-    case EPI_RICH_ADDX: x[o] += (double)(t + (MT)in[o]); break;
-    case EPI_RICH_SETX: x[o] = (double)(t + (MT)in[o]); break;
-    case EPI_SPMV: st_keep(out + o, (VO)t, keep); break;
-    default: break;
-  }
 }
 
 // R interleaved right-hand sides, one lane per row: acc[k] -/+= sum v[p]
@@ -807,7 +646,7 @@ __global__ void __launch_bounds__(W * 32, 1)
     const int r = dcur.x + lane;
     const bool act = r < dcur.y;
     MT acc = (act && c) ? (MT)ld_keep(c + r, keep) : MT(0);
-    if (act) prefetch_epilogue(epi, r, dinv, x);
+    if (act) prefetch_epilogue(epi, r, (size_t)r, dinv, x);
     const int s = k % kWarpStages;
     const bool ok = mbar_wait_bounded(&full[warp][s], (uint32_t)(k / kWarpStages) & 1u);
     if (!__all_sync(0xffffffffu, ok)) {

@@ -104,6 +104,11 @@ void solve_one(silu_server S, silu_ctx ctx, const std::shared_ptr<Request>& r) {
   double* db = nullptr;
   int status = SILU_OK;
   const int64_t n = q.A.n;
+  // one device copy of each matrix, as the memory estimate counts them; exact
+  // solves read the factors' CSR arrays
+  const bool direct = q.p.precond == SILU_PRECOND_DIRECT || q.p.precond == SILU_PRECOND_AMG_DIRECT;
+  ctx->copies = Copies::kSmaller;
+  ctx->factor_copies = direct ? Copies::kCsr : Copies::kSmaller;
   do {
     status = silu_mat_create(ctx, n, q.A.nnz(), q.A.rp.data(), q.A.ci.data(), q.A.va.data(), &M);
     if (status != SILU_OK) break;

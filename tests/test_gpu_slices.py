@@ -1,0 +1,151 @@
+"""The sliced sweep (the default path of every product and sweep): sizes
+around a slice of 32 rows, 16-bit and int32 columns, one to five interleaved
+right-hand sides at 16- and 8-byte alignment, padding next to infinite
+entries, and new values after a refactorisation."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+from _helpers import maxabs_err, relerr
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+FP64_TOL = 1e-12
+
+
+@pytest.fixture(scope="module")
+def silu():
+    import paper_2111_09512_gb300 as s
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    s.build()
+    return s
+
+
+@pytest.fixture(scope="module")
+def ctx(silu):
+    return silu.Context(0, torch.cuda.current_stream())
+
+
+def dev(a, shift=0):
+    """A contiguous device copy whose address is 8 * shift bytes past a 256-byte boundary."""
+    a = np.ascontiguousarray(a)
+    buf = torch.empty(a.size + shift, dtype=torch.float64, device="cuda")
+    t = buf[shift:].view(a.shape)
+    t.copy_(torch.from_numpy(a))
+    return t
+
+
+def host(t):
+    torch.cuda.synchronize()
+    return t.cpu().numpy()
+
+
+def far(n, reach):
+    """Tridiagonal plus couplings `reach` rows away (diagonally dominant)."""
+    i = np.arange(n)
+    rows, cols = [i], [i]
+    for d in (1, reach):
+        rows += [i[d:], i[:-d]]
+        cols += [i[:-d], i[d:]]
+    r, c = np.concatenate(rows), np.concatenate(cols)
+    order = np.lexsort((c, r))
+    r, c = r[order], c[order]
+    v = np.where(r == c, 5.0, -synth.uniform(5, 1, len(r), 0.1, 1.0))
+    rp = np.zeros(n + 1, np.int64)
+    np.add.at(rp, r + 1, 1)
+    return np.cumsum(rp), c.astype(np.int32), v
+
+
+CASES = [
+    ("1 row", lambda: synth.banded(1, 0, 1, seed=12)),
+    ("31 rows", lambda: synth.banded(31, 5, 31, seed=11)),
+    ("32 rows", lambda: synth.banded(32, 4, 12, seed=3)),
+    ("33 rows", lambda: synth.banded(33, 3, 8, seed=10)),
+    ("cutcell 37x29x23", lambda: synth.cutcell7(37, 29, 23, seed=1)),
+    ("hex27 17x13x11", lambda: synth.hex27(17, 13, 11, seed=3)),
+    ("columns 65534 apart", lambda: far(65600, 65534 // 2 - 16)),
+    ("columns beyond 16 bits", lambda: far(66100, 66001)),
+]
+
+
+@pytest.mark.parametrize("shift", [0, 1], ids=["aligned", "odd"])
+@pytest.mark.parametrize("case", CASES, ids=[c[0] for c in CASES])
+def test_sliced_products_and_sweeps_match_oracle(silu, ctx, case, shift):
+    A = case[1]()
+    n = len(A[0]) - 1
+    M = silu.Matrix(ctx, *A)
+    F = silu.ilu_setup(ctx, M, "ilu0")
+    F.set_fused(1)
+    F32 = silu.ilu_setup(ctx, M, "ilu0", prec=silu.FP32)
+    F32.set_fused(1)
+    S = oracle.row_scale(oracle.factor(A, "ilu0", 0.0, 0))
+    for nrhs in (1, 2, 3, 4, 5):
+        b, x0 = synth.rhs(n, nrhs, seed=21), synth.rhs(n, nrhs, seed=22) * 0.5
+        r = dev(np.zeros((n, nrhs)), shift)
+        M.residual(r, dev(x0, shift), dev(b, shift))
+        assert maxabs_err(host(r), oracle.residual(A, x0, b)) < FP64_TOL, nrhs
+        for mL, mU in [(3, 4), (1, 1), (2, 0)]:
+            want = oracle.smooth(A, S, x0, b, mL, mU)
+            for G, tol in ((F, FP64_TOL), (F32, 1e-5)):
+                x = dev(x0, shift)
+                silu.ilu_smooth(G, x, dev(b, shift), mL, mU)
+                ctx.check()
+                got = host(x)
+                for k in range(nrhs):
+                    assert relerr(got[:, k], want[:, k]) < tol, (nrhs, mL, mU, k)
+
+
+@pytest.mark.parametrize("name,gen", [CASES[4], CASES[7]], ids=[CASES[4][0], CASES[7][0]])
+def test_sliced_sweeps_give_the_tiled_sweeps_bits(silu, ctx, name, gen):
+    """One lane sums a row in column order on slices as on tiles."""
+    A = gen()
+    n = len(A[0]) - 1
+    b, x0 = synth.rhs(n, 1, seed=1), synth.rhs(n, 1, seed=2)
+    for prec in (silu.FP64, silu.FP32):
+        F = silu.ilu_setup(ctx, silu.Matrix(ctx, *A), "ilut", 1e-3, 10, prec=prec)
+        out = []
+        for variant in (0, 2):
+            F.set_kernel(variant)
+            x = dev(x0)
+            silu.ilu_smooth(F, x, dev(b), 6, 5)
+            out.append(host(x))
+        assert np.array_equal(out[0], out[1])
+
+
+def test_padding_reads_no_vector_entry(silu, ctx):
+    """An infinite or NaN entry of x reaches only the rows that refer to it."""
+    A = synth.cutcell7(21, 17, 13, seed=5)
+    n = len(A[0]) - 1
+    rp, ci, _ = A
+    b, x = synth.rhs(n, 1, seed=3), synth.rhs(n, 1, seed=4)
+    clean = oracle.residual(A, x, b)[:, 0]
+    M = silu.Matrix(ctx, *A)
+    for j, bad in ((0, np.inf), (n // 2, np.nan), (n - 1, -np.inf)):
+        xb = x.copy()
+        xb[j] = bad
+        r = dev(np.zeros((n, 1)))
+        M.residual(r, dev(xb), dev(b))
+        got = host(r)[:, 0]
+        hit = np.zeros(n, bool)
+        for i in range(n):
+            hit[i] = j in ci[rp[i]:rp[i + 1]]
+        assert not np.isfinite(got[hit]).any() and relerr(got[~hit], clean[~hit]) < FP64_TOL
+
+
+def test_refactor_renews_the_slices_of_the_matrix(silu, ctx):
+    A, A2 = synth.cutcell7(19, 18, 17, seed=3), synth.cutcell7(19, 18, 17, seed=8)
+    n = len(A[0]) - 1
+    M = silu.Matrix(ctx, *A)
+    F = silu.ilu_setup(ctx, M, "ilu0")
+    silu.ilu_refactor(F, A2[2])
+    b, x0 = synth.rhs(n, 1, seed=5), synth.rhs(n, 1, seed=6)
+    S = oracle.row_scale(oracle.factor(A2, "ilu0", 0.0, 0))
+    x = dev(x0)
+    silu.ilu_smooth(F, x, dev(b), 4, 4)
+    assert relerr(host(x), oracle.smooth(A2, S, x0, b, 4, 4)) < FP64_TOL
+    r = dev(np.zeros((n, 1)))
+    M.residual(r, dev(x0), dev(b))
+    assert relerr(host(r), oracle.residual(A2, x0, b)) < FP64_TOL
