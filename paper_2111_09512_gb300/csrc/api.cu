@@ -240,6 +240,8 @@ cudaError_t allocate_krylov(silu_ilu F, int m) {
   if ((e = w.part0.ensure(sizeof(double) * 1024)) != cudaSuccess) return e;
   if ((e = w.part1.ensure(sizeof(double) * 1024)) != cudaSuccess) return e;
   if ((e = w.scal.ensure(sizeof(double) * 8)) != cudaSuccess) return e;
+  if ((e = w.arn.ensure(silu::arnoldi_bytes((int)n))) != cudaSuccess) return e;
+  if ((e = cudaMemsetAsync(w.arn.p, 0, w.arn.bytes, F->ctx->stream)) != cudaSuccess) return e;
   w.restart = m;
   return cudaSuccess;
 }
@@ -881,6 +883,12 @@ void fgmres_inner(silu_ilu F, int j, int m, int mL, int mU, int precond, bool ca
   else
     CK(cudaMemcpyAsync(zj, vj, sizeof(double) * (size_t)n, cudaMemcpyDeviceToDevice, s));
   LAUNCH(F->ctx, SILU_K_RESIDUAL, sweep_launch(F, F->A->d, silu::MODE_D, 1, gA, 1, nullptr, zj, w, nullptr, nullptr, silu::EPI_SPMV));
+  if (silu::arnoldi_fits(n, m, F->ctx->env)) {
+    LAUNCH(F->ctx, SILU_K_KRYLOV,
+           silu::launch_arnoldi(n, j, m, w, V, H, W.cs.as<double>(), W.sn.as<double>(), W.g.as<double>(),
+                                W.scal.as<double>() + 1, W.arn.p, F->ctx->env, s));
+    return;
+  }
   LAUNCH(F->ctx, SILU_K_KRYLOV, silu::launch_dot_part(n, w, V, part[0], s));
   int cur = 0;
   for (int i = 0; i <= j; ++i) {
@@ -888,8 +896,9 @@ void fgmres_inner(silu_ilu F, int j, int m, int mL, int mU, int precond, bool ca
     LAUNCH(F->ctx, SILU_K_KRYLOV, silu::launch_mgs_step(n, part[cur], H + (size_t)i * m + j, w, vec(V, i), vnext, part[cur ^ 1], s));
     cur ^= 1;
   }
-  LAUNCH(F->ctx, SILU_K_KRYLOV, silu::launch_normalize(n, part[cur], H + (size_t)(j + 1) * m + j, w, vec(V, j + 1), s));
-  LAUNCH(F->ctx, SILU_K_KRYLOV, silu::launch_givens(j, m, H, W.cs.as<double>(), W.sn.as<double>(), W.g.as<double>(), W.scal.as<double>() + 1, s));
+  LAUNCH(F->ctx, SILU_K_KRYLOV,
+         silu::launch_normalize_givens(n, part[cur], w, vec(V, j + 1), j, m, H, W.cs.as<double>(), W.sn.as<double>(),
+                                       W.g.as<double>(), W.scal.as<double>() + 1, s));
 }
 
 // Run inner iteration j from its captured graph (capturing it on first use).
@@ -1016,6 +1025,7 @@ silu_status silu_ctx_create(int device, void* cuda_stream, silu_ctx* out) {
     if (e == cudaSuccess) e = cudaMemset(c->env.err, 0, 4 * sizeof(int));
     if (e == cudaSuccess) e = silu::staged_prepare();
     if (e == cudaSuccess) e = silu::slices_prepare();
+    if (e == cudaSuccess) e = silu::arnoldi_prepare(c->env);
     if (e != cudaSuccess) {
       delete c;
       return SILU_ERR_CUDA;

@@ -166,9 +166,12 @@ struct LaunchEnv {
   int* err = nullptr;   // err[0]: device error word (bit 0: a copy wait gave up,
                         // bit 1: the self-test wait gave up, bit 2: a wait of
                         // the persistent triangular solve gave up, bit 3: a
-                        // grid barrier of the fused smoother gave up); err[1]:
+                        // grid barrier of the fused smoother gave up, bit 4: an
+                        // exchange of an Arnoldi step gave up); err[1]:
                         // a flag that nothing sets (self-test); err[2..3]: the
                         // fused smoother's grid-barrier words
+  bool arnoldi = false;     // the blocks of the one-launch Arnoldi step fit on a multiprocessor
+  int arnoldi_cluster = 0;  // largest cluster of its small form that fits on the device
   bool overlap = true;  // staged sweeps launched as programmatic dependents of
                         // the kernel before them (prologue overlaps its tail)
   int l2 = kL2Default;  // L2 reuse flags of staged sweeps (kFlag* above)

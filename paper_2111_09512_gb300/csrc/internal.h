@@ -124,7 +124,7 @@ struct Workspace {
     kgraphs.clear();
   }
   int restart = 0;
-  DBuf V, Z, w, H, cs, sn, g, yk, part0, part1, scal;
+  DBuf V, Z, w, H, cs, sn, g, yk, part0, part1, scal, arn;
 };
 
 // Device arrays of a length-sorted copy of a factor (staged kernel only).

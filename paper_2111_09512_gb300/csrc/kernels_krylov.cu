@@ -15,6 +15,7 @@ namespace {
 
 constexpr int KB = 256;
 constexpr int kMaxParts = 1024;
+constexpr int kGivensStaged = 1024;  // columns whose Givens update fits in shared memory without opting in
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -130,6 +131,62 @@ __global__ void __launch_bounds__(KB, 8) k_normalize(int n, const double* __rest
   for (; i < N; i += S) vout[i] = w[i] / h;
 }
 
+// The end of Arnoldi step j: h_{j+1,j} and v_{j+1} as k_normalize, and, by one
+// thread of block 0, the Givens update of column j (the rows h_0 .. h_j of H):
+// the earlier rotations, the new one, the right-hand side g.  Column and
+// rotations are read by the whole block first: the update is a chain of
+// dependent operations, and reading each operand from memory where it is used
+// took 10 us at j = 16.
+__global__ void __launch_bounds__(KB, 8) k_normalize_givens(int n, const double* __restrict__ part_in, int nparts,
+                                                            const double* w, double* vout, int j, int m, double* H,
+                                                            double* cs, double* sn, double* g, double* res) {
+  extern __shared__ double sh[];  // block 0: column j (j + 1 entries), cs and sn (j each); none where that is too much
+  const bool lead = blockIdx.x == 0;
+  const bool staged = j < kGivensStaged;
+  double* col = staged ? sh : H + j;  // entry i at col[i * ld]
+  const size_t ld = staged ? 1 : (size_t)m;
+  const double* c0 = staged ? sh + j + 1 : cs;
+  const double* s0 = staged ? sh + 2 * j + 1 : sn;
+  if (lead && staged) {
+    for (int i = threadIdx.x; i <= j; i += KB) sh[i] = H[(size_t)i * m + j];
+    for (int i = threadIdx.x; i < j; i += KB) {
+      sh[j + 1 + i] = cs[i];
+      sh[2 * j + 1 + i] = sn[i];
+    }
+  }
+  const double h = sqrt(sum_parts(part_in, nparts));
+  if (h != 0.0) {
+    const unsigned N = (unsigned)n, S = gridDim.x * KB;
+    unsigned i = blockIdx.x * KB + threadIdx.x;
+    for (; i + S < N; i += 2 * S) {
+      const double w0 = w[i], w1 = w[i + S];
+      vout[i] = w0 / h;
+      vout[i + S] = w1 / h;
+    }
+    for (; i < N; i += S) vout[i] = w[i] / h;
+  }
+  if (!lead || threadIdx.x != 0) return;
+  for (int i = 0; i < j; ++i) {
+    const double a = col[i * ld], b = col[(i + 1) * ld];
+    const double c = c0[i], s = s0[i];
+    H[(size_t)i * m + j] = c * a + s * b;
+    col[(i + 1) * ld] = -s * a + c * b;
+  }
+  const double a = col[j * ld], b = h;
+  const double den = hypot(a, b);
+  const double c = den != 0.0 ? a / den : 1.0;
+  const double s = den != 0.0 ? b / den : 0.0;
+  cs[j] = c;
+  sn[j] = s;
+  H[(size_t)j * m + j] = den;
+  H[(size_t)(j + 1) * m + j] = 0.0;
+  const double gj = g[j];
+  g[j + 1] = -s * gj;
+  g[j] = c * gj;
+  res[0] = fabs(-s * gj);
+  res[1] = b;  // h_{j+1,j}: zero means the Krylov space is exhausted
+}
+
 // Minimal-residual step: alpha = sum(part_num) / sum(part_den) (0 when the
 // denominator is 0), y = alpha s.
 __global__ void __launch_bounds__(KB) k_mr_step(int n, const double* __restrict__ part_num,
@@ -145,29 +202,6 @@ __global__ void __launch_bounds__(KB) k_mr_step(int n, const double* __restrict_
 __global__ void k_norm_final(const double* __restrict__ part_in, int nparts, double* __restrict__ out) {
   const double h = sqrt(sum_parts(part_in, nparts));
   if (threadIdx.x == 0) *out = h;
-}
-
-// One thread: apply the earlier rotations to column j, make the new one,
-// rotate g (right-hand side of the least-squares problem).
-__global__ void k_givens(int j, int m, double* H, double* cs, double* sn, double* g, double* res) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  for (int i = 0; i < j; ++i) {
-    const double a = H[i * m + j], b = H[(i + 1) * m + j];
-    H[i * m + j] = cs[i] * a + sn[i] * b;
-    H[(i + 1) * m + j] = -sn[i] * a + cs[i] * b;
-  }
-  const double a = H[j * m + j], b = H[(j + 1) * m + j];
-  const double den = hypot(a, b);
-  const double c = den != 0.0 ? a / den : 1.0;
-  const double s = den != 0.0 ? b / den : 0.0;
-  cs[j] = c;
-  sn[j] = s;
-  H[j * m + j] = den;
-  H[(j + 1) * m + j] = 0.0;
-  g[j + 1] = -s * g[j];
-  g[j] = c * g[j];
-  res[0] = fabs(g[j + 1]);
-  res[1] = b;  // h_{j+1,j}: zero means the Krylov space is exhausted
 }
 
 // Every block solves the small triangle (redundantly, same order) and then
@@ -221,6 +255,15 @@ cudaError_t launch_normalize(int n, const double* part_in, double* hout, const d
   return cudaGetLastError();
 }
 
+cudaError_t launch_normalize_givens(int n, const double* part_in, const double* w, double* vout, int j, int m,
+                                    double* H, double* cs, double* sn, double* g, double* res, cudaStream_t s) {
+  const int np = krylov_parts(n);
+  const size_t smem = j < kGivensStaged ? sizeof(double) * (size_t)(3 * j + 1) : 0;
+  k_normalize_givens<<<np, KB, smem, s>>>(n, part_in, np, w, vout, j, m, H, cs, sn, g,
+                                                                         res);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_mr_step(int n, const double* part_num, const double* part_den, const double* sv, double* y,
                            cudaStream_t s) {
   const int np = krylov_parts(n);
@@ -230,11 +273,6 @@ cudaError_t launch_mr_step(int n, const double* part_num, const double* part_den
 
 cudaError_t launch_norm_final(int n, const double* part_in, double* out, cudaStream_t s) {
   k_norm_final<<<1, KB, 0, s>>>(part_in, krylov_parts(n), out);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_givens(int j, int m, double* H, double* cs, double* sn, double* g, double* res, cudaStream_t s) {
-  k_givens<<<1, 32, 0, s>>>(j, m, H, cs, sn, g, res);
   return cudaGetLastError();
 }
 
