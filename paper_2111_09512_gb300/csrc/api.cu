@@ -893,7 +893,8 @@ void fgmres_inner(silu_ilu F, int j, int m, int mL, int mU, int precond, bool ca
   int cur = 0;
   for (int i = 0; i <= j; ++i) {
     const double* vnext = (i < j) ? vec(V, i + 1) : nullptr;
-    LAUNCH(F->ctx, SILU_K_KRYLOV, silu::launch_mgs_step(n, part[cur], H + (size_t)i * m + j, w, vec(V, i), vnext, part[cur ^ 1], s));
+    LAUNCH(F->ctx, SILU_K_KRYLOV, silu::launch_mgs_step(n, part[cur], H + (size_t)i * m + j, w, vec(V, i), vnext, part[cur ^ 1],
+                                                          F->ctx->env.sms, s));
     cur ^= 1;
   }
   LAUNCH(F->ctx, SILU_K_KRYLOV,

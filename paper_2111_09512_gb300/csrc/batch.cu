@@ -14,6 +14,7 @@
 // number of systems still active.
 #include <thread>
 
+#include "exchange.cuh"
 #include "internal.h"
 
 using namespace silu;
@@ -51,10 +52,18 @@ __device__ double block_sum(double v) {
 // Sum of system s's chunk partials, in chunk order (thread 0), broadcast.
 __device__ double system_sum(const double* __restrict__ part, const int* __restrict__ sys_chunk0, int s) {
   __shared__ double v;
-  if (threadIdx.x == 0) {
+  // the partials by a warp, up to 64 at once; the adds are a serial chain
+  if (threadIdx.x < 32) {
     double a = 0.0;
-    for (int c = sys_chunk0[s]; c < sys_chunk0[s + 1]; ++c) a += part[c];
-    v = a;
+    const int c1 = sys_chunk0[s + 1];
+    for (int c = sys_chunk0[s]; c < c1; c += 64) {
+      const int l = threadIdx.x;
+      const double p0 = c + l < c1 ? part[c + l] : 0.0, p1 = c + 32 + l < c1 ? part[c + 32 + l] : 0.0;
+      const int n0 = min(32, c1 - c), n1 = min(32, c1 - c - 32);
+      for (int q = 0; q < n0; ++q) a += __shfl_sync(0xffffffffu, p0, q);
+      for (int q = 0; q < n1; ++q) a += __shfl_sync(0xffffffffu, p1, q);
+    }
+    if (threadIdx.x == 0) v = a;
   }
   __syncthreads();
   const double out = v;
@@ -87,7 +96,14 @@ __global__ void __launch_bounds__(KB, 8) k_bdot(int nch, const int4* __restrict_
 // MGS step i of Arnoldi column j for every active system:
 //   h = <w, v_i>_s (from part_in);  H_s[i][j] = h;  w -= h v_i;
 //   part_out = chunk partials of <w, v_next> (or |w|^2 when v_next is null).
-__global__ void __launch_bounds__(KB, 8) k_bmgs(int nch, const int4* __restrict__ ch, const int* __restrict__ sys_chunk0,
+// U rows are loaded at a time; with U = 4 a chunk's first ones before h is
+// summed: with one block per chunk (up to four per SM) a step is the latency
+// of its loads and of the serial sum of the system's partials, not bandwidth.
+// U = 2 for larger grids, which want eight blocks per SM.  Keeping w in
+// registers through all steps of a column (one launch, partials exchanged
+// through L2) was slower: 24.5 us per step at any number of systems.
+template <int U>
+__global__ void __launch_bounds__(KB, U > 2 ? 4 : 8) k_bmgs(int nch, const int4* __restrict__ ch, const int* __restrict__ sys_chunk0,
                                              const double* __restrict__ part_in, double* __restrict__ H, int m,
                                              int i, int j, double* __restrict__ w, const double* __restrict__ vi,
                                              const double* __restrict__ vnext, double* __restrict__ part_out,
@@ -99,33 +115,32 @@ __global__ void __launch_bounds__(KB, 8) k_bmgs(int nch, const int4* __restrict_
       if (threadIdx.x == 0) part_out[c] = 0.0;
       continue;
     }
+    int r = d.y + threadIdx.x;
+    double w0[U], v0[U], u0[U];
+    auto load = [&]() {
+#pragma unroll
+      for (int k = 0; k < U; ++k) {
+        const bool in = r + k * KB < d.z;
+        w0[k] = in ? w[r + k * KB] : 0.0;
+        v0[k] = in ? vi[r + k * KB] : 0.0;
+        u0[k] = in && vnext ? vnext[r + k * KB] : 0.0;
+      }
+    };
+    if constexpr (U > 2) load();
     const double h = system_sum(part_in, sys_chunk0, s);
     if (threadIdx.x == 0 && c == sys_chunk0[s]) H[((size_t)s * (m + 1) + i) * m + j] = h;
+    if constexpr (U <= 2) load();
     double acc = 0.0;
-    int r = d.y + threadIdx.x;
-    if (vnext) {
-      for (; r + KB < d.z; r += 2 * KB) {
-        const double w0 = w[r], w1 = w[r + KB], v0 = vi[r], v1 = vi[r + KB], u0 = vnext[r], u1 = vnext[r + KB];
-        const double n0 = w0 - h * v0, n1 = w1 - h * v1;
-        w[r] = n0;
-        w[r + KB] = n1;
-        acc += n0 * u0;
-        acc += n1 * u1;
-      }
-    } else {
-      for (; r + KB < d.z; r += 2 * KB) {
-        const double w0 = w[r], w1 = w[r + KB], v0 = vi[r], v1 = vi[r + KB];
-        const double n0 = w0 - h * v0, n1 = w1 - h * v1;
-        w[r] = n0;
-        w[r + KB] = n1;
-        acc += n0 * n0;
-        acc += n1 * n1;
-      }
-    }
-    for (; r < d.z; r += KB) {
-      const double wn = w[r] - h * vi[r];
-      w[r] = wn;
-      acc += wn * (vnext ? vnext[r] : wn);
+    while (r < d.z) {
+#pragma unroll
+      for (int k = 0; k < U; ++k)
+        if (r + k * KB < d.z) {
+          const double wn = w0[k] - h * v0[k];
+          w[r + k * KB] = wn;
+          acc += wn * (vnext ? u0[k] : wn);
+        }
+      r += U * KB;
+      if (r < d.z) load();
     }
     const double t = block_sum(acc);
     if (threadIdx.x == 0) part_out[c] = t;
@@ -133,7 +148,7 @@ __global__ void __launch_bounds__(KB, 8) k_bmgs(int nch, const int4* __restrict_
 }
 
 // h = sqrt(<w, w>_s); H_s[j+1][j] = h; v_{j+1} = w / h (active systems, h != 0)
-__global__ void __launch_bounds__(KB, 8) k_bnormalize(int nch, const int4* __restrict__ ch,
+__global__ void __launch_bounds__(KB, 5) k_bnormalize(int nch, const int4* __restrict__ ch,
                                                    const int* __restrict__ sys_chunk0,
                                                    const double* __restrict__ part_in, double* __restrict__ H, int m,
                                                    int j, const double* __restrict__ w, double* __restrict__ vout,
@@ -145,13 +160,14 @@ __global__ void __launch_bounds__(KB, 8) k_bnormalize(int nch, const int4* __res
     const double h = sqrt(system_sum(part_in, sys_chunk0, s));
     if (threadIdx.x == 0 && c == sys_chunk0[s]) H[((size_t)s * (m + 1) + j + 1) * m + j] = h;
     if (h == 0.0) continue;
+    const Divider by(h);
     int r = d.y + threadIdx.x;
     for (; r + KB < d.z; r += 2 * KB) {
       const double w0 = w[r], w1 = w[r + KB];
-      vout[r] = w0 / h;
-      vout[r + KB] = w1 / h;
+      vout[r] = by(w0);
+      vout[r + KB] = by(w1);
     }
-    for (; r < d.z; r += KB) vout[r] = w[r] / h;
+    for (; r < d.z; r += KB) vout[r] = by(w[r]);
   }
 }
 
@@ -196,48 +212,58 @@ __global__ void k_bstart(int ns, int m, const double* __restrict__ beta, const d
   }
 }
 
-// Givens step j, one block, one thread per system.
+// Givens step j, a warp per system: the lanes read the column and the
+// rotations (up to 32 of each at a time), then all apply the same rotations in
+// registers, a chain of dependent operations that one thread per system ran
+// through memory (17 us at 24 systems).  Blocks of 8 warps; *count, zero
+// before the launch, becomes the number of systems still active.
 __global__ void k_bgivens(int ns, int j, int m, double* __restrict__ H, double* __restrict__ cs, double* __restrict__ sn,
                           double* __restrict__ g, const double* __restrict__ bnorm, double tol, int maxit,
                           int* __restrict__ act, int* __restrict__ its, int* __restrict__ jend,
                           int* __restrict__ count) {
-  __shared__ int cnt[KB];
-  int mine = 0;
-  for (int s = threadIdx.x; s < ns; s += blockDim.x) {
-    if (!act[s]) continue;
-    double* Hs = H + (size_t)s * (m + 1) * m;
-    double* cs_s = cs + (size_t)s * m;
-    double* sn_s = sn + (size_t)s * m;
-    double* gs = g + (size_t)s * (m + 1);
-    for (int i = 0; i < j; ++i) {
-      const double a = Hs[i * m + j], b = Hs[(i + 1) * m + j];
-      Hs[i * m + j] = cs_s[i] * a + sn_s[i] * b;
-      Hs[(i + 1) * m + j] = -sn_s[i] * a + cs_s[i] * b;
+  const int s = blockIdx.x * (KB / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (s >= ns || !act[s]) return;
+  double* Hs = H + (size_t)s * (m + 1) * m;
+  double* cs_s = cs + (size_t)s * m;
+  double* sn_s = sn + (size_t)s * m;
+  double* gs = g + (size_t)s * (m + 1);
+  double a = Hs[j];  // entry i of the column as the earlier rotations leave it
+  for (int i0 = 0; i0 < j; i0 += 32) {
+    const int i = i0 + lane;
+    const double bl = i < j ? Hs[(size_t)(i + 1) * m + j] : 0.0;
+    const double cl = i < j ? cs_s[i] : 0.0, sl = i < j ? sn_s[i] : 0.0;
+    double keep = 0.0;
+    const int nq = min(32, j - i0);
+    for (int q = 0; q < nq; ++q) {
+      const double b = __shfl_sync(0xffffffffu, bl, q);
+      const double c = __shfl_sync(0xffffffffu, cl, q), sv = __shfl_sync(0xffffffffu, sl, q);
+      const double top = c * a + sv * b;
+      if (lane == q) keep = top;
+      a = -sv * a + c * b;
     }
-    const double a = Hs[j * m + j], b = Hs[(j + 1) * m + j];
-    const double hnext = b;
-    const double den = hypot(a, b);
-    const double c = den != 0.0 ? a / den : 1.0;
-    const double sgn = den != 0.0 ? b / den : 0.0;
-    cs_s[j] = c;
-    sn_s[j] = sgn;
-    Hs[j * m + j] = den;
-    Hs[(j + 1) * m + j] = 0.0;
-    gs[j + 1] = -sgn * gs[j];
-    gs[j] = c * gs[j];
-    its[s] += 1;
-    jend[s] = j + 1;
-    const bool stop = fabs(gs[j + 1]) <= tol * bnorm[s] || its[s] >= maxit || hnext == 0.0 || !isfinite(gs[j + 1]);
-    if (stop) act[s] = 0;
-    mine += stop ? 0 : 1;
+    if (i < j) Hs[(size_t)i * m + j] = keep;
   }
-  cnt[threadIdx.x] = mine;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int t = 0;
-    for (int k = 0; k < blockDim.x; ++k) t += cnt[k];
-    *count = t;
-  }
+  if (lane != 0) return;
+  const double b = Hs[(size_t)(j + 1) * m + j];
+  const double hnext = b;
+  const double den = hypot(a, b);
+  const double c = den != 0.0 ? a / den : 1.0;
+  const double sgn = den != 0.0 ? b / den : 0.0;
+  cs_s[j] = c;
+  sn_s[j] = sgn;
+  Hs[(size_t)j * m + j] = den;
+  Hs[(size_t)(j + 1) * m + j] = 0.0;
+  const double gj = gs[j], gn = -sgn * gj;
+  gs[j + 1] = gn;
+  gs[j] = c * gj;
+  const int it = its[s] + 1;
+  its[s] = it;
+  jend[s] = j + 1;
+  const bool stop = fabs(gn) <= tol * bnorm[s] || it >= maxit || hnext == 0.0 || !isfinite(gn);
+  if (stop)
+    act[s] = 0;
+  else
+    atomicAdd(count, 1);
 }
 
 // x_s += Z y_s with H_s y_s = g_s (jend_s x jend_s triangle), every system
@@ -277,8 +303,8 @@ __global__ void __launch_bounds__(KB) k_bdivide(int nch, const int4* __restrict_
     const int4 d = ch[c];
     const int s = d.x;
     if (!act[s] || scal[s] == 0.0) continue;
-    const double q = scal[s];
-    for (int r = d.y + threadIdx.x; r < d.z; r += KB) out[r] = in[r] / q;
+    const Divider by(scal[s]);
+    for (int r = d.y + threadIdx.x; r < d.z; r += KB) out[r] = by(in[r]);
   }
 }
 
@@ -386,8 +412,8 @@ void inner_iteration(silu_batch B, int j, int m, int mL, int mU, int precond, do
   for (int i = 0; i <= j; ++i) {
     const double* vnext = (i < j) ? V + (size_t)(i + 1) * N : nullptr;
     LAUNCH(ctx, SILU_K_KRYLOV,
-           (k_bmgs<<<grid, KB, 0, s>>>(B->nch, ch, sc0, part[cur], B->H.as<double>(), m, i, j, w, V + (size_t)i * N,
-                                        vnext, part[cur ^ 1], act),
+           ((grid <= 4 * ctx->env.sms ? k_bmgs<4> : k_bmgs<2>)<<<grid, KB, 0, s>>>(
+                B->nch, ch, sc0, part[cur], B->H.as<double>(), m, i, j, w, V + (size_t)i * N, vnext, part[cur ^ 1], act),
             cudaGetLastError()));
     cur ^= 1;
   }
@@ -395,8 +421,9 @@ void inner_iteration(silu_batch B, int j, int m, int mL, int mU, int precond, do
          (k_bnormalize<<<grid, KB, 0, s>>>(B->nch, ch, sc0, part[cur], B->H.as<double>(), m, j, w,
                                            V + (size_t)(j + 1) * N, act),
           cudaGetLastError()));
+  CK(cudaMemsetAsync(B->counter.as<int>() + 1, 0, sizeof(int), s));
   LAUNCH(ctx, SILU_K_KRYLOV,
-         (k_bgivens<<<1, KB, 0, s>>>(B->count, j, m, B->H.as<double>(), B->cs.as<double>(), B->sn.as<double>(),
+         (k_bgivens<<<(B->count + KB / 32 - 1) / (KB / 32), KB, 0, s>>>(B->count, j, m, B->H.as<double>(), B->cs.as<double>(), B->sn.as<double>(),
                                      B->g.as<double>(), B->bnorm.as<double>(), tol, maxit, B->act.as<int>(),
                                      B->its.as<int>(), B->jend.as<int>(), B->counter.as<int>() + 1),
           cudaGetLastError()));
@@ -618,6 +645,7 @@ silu_status silu_batch_fgmres(silu_batch B, double* x, const double* b, double t
   try {
     CK(ensure_vectors(F, 1));
     CK(ensure_bkrylov(B, m));
+
     // captured iterations carry tol and maxit as kernel arguments
     if (tol != B->graph_tol || maxit != B->graph_maxit) {
       for (InnerGraph& ig : B->graphs)

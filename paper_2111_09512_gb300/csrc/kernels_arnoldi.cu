@@ -37,6 +37,7 @@
 #include <cmath>
 
 #include "device.cuh"
+#include "exchange.cuh"
 #include "krylov.cuh"
 
 namespace silu {
@@ -45,60 +46,6 @@ namespace {
 constexpr int kArnRows = 8;  // rows per thread at most
 constexpr int kArnMaxBasis = 1024;
 constexpr int kArnMaxGroups = 512;
-constexpr unsigned long long kArnWaitNs = 2000000000ull;
-
-__device__ __forceinline__ unsigned long long arn_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
-__device__ __forceinline__ double arn_warp_sum(double v) {
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-  return v;
-}
-
-__device__ __forceinline__ void publish(ulonglong2* e, double v, unsigned tag) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-  const unsigned long long t = (unsigned long long)tag << 32;
-  const unsigned long long lo = t | (b & 0xffffffffull), hi = t | (b >> 32);
-  asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(e), "l"(lo), "l"(hi) : "memory");
-}
-
-__device__ __forceinline__ bool peek(const ulonglong2* e, unsigned tag, double& v) {
-  unsigned long long lo, hi;
-  asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(lo), "=l"(hi) : "l"(e) : "memory");
-  if ((unsigned)(lo >> 32) != tag || (unsigned)(hi >> 32) != tag) return false;
-  v = __longlong_as_double((long long)((hi << 32) | (lo & 0xffffffffull)));
-  return true;
-}
-
-// The K values at e[0], e[stride], ... (those with k < cnt), once all are there.
-template <int K>
-__device__ __forceinline__ void collect(const ulonglong2* e, int stride, int cnt, unsigned tag, double (&v)[K],
-                                        bool& alive, int* err) {
-  unsigned missing = 0;
-#pragma unroll
-  for (int k = 0; k < K; ++k) {
-    v[k] = 0.0;
-    if (k < cnt && !peek(e + k * stride, tag, v[k])) missing |= 1u << k;
-  }
-  if (!missing || !alive) return;
-  const unsigned long long t0 = arn_ns();
-  for (unsigned spins = 1; missing; ++spins) {
-    __nanosleep(100);
-#pragma unroll
-    for (int k = 0; k < K; ++k)
-      if ((missing >> k) & 1u)
-        if (peek(e + k * stride, tag, v[k])) missing &= ~(1u << k);
-    if ((spins & 255u) == 0 && arn_ns() - t0 > kArnWaitNs) {
-      atomicOr(err, 16);
-      alive = false;
-      return;
-    }
-  }
-}
 
 struct ArnoldiArgs {
   int n, np, j, m;
@@ -214,10 +161,11 @@ struct ArnoldiRows {
   }
   __device__ __forceinline__ void normalize(double h, double* vout) const {
     if (h == 0.0) return;
+    const Divider by(h);
     vout += i0;
 #pragma unroll
     for (int k = 0; k < kArnRows; ++k)
-      if (k < cnt) vout[(size_t)k * S] = w[k] / h;
+      if (k < cnt) vout[(size_t)k * S] = by(w[k]);
   }
 };
 

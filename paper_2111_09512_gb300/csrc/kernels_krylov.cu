@@ -8,6 +8,7 @@
 #include <cmath>
 
 #include "device.cuh"
+#include "exchange.cuh"
 #include "krylov.cuh"
 
 namespace silu {
@@ -71,46 +72,42 @@ __global__ void __launch_bounds__(KB, 8) k_dot_part(int n, const double* __restr
   if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
 
-__global__ void __launch_bounds__(KB, 8) k_mgs_step(int n, const double* __restrict__ part_in, int nparts,
+// U rows are loaded at a time.  U = 4, the first ones before h is summed, for
+// grids of at most four blocks per SM, where a step is the latency of its
+// loads (FGMRES, 60 iterations: Poisson 48^3 / 64^3 7264 / 8582 -> 7001 / 8285
+// us); U = 2 (32 registers, eight blocks per SM) beyond, where it is bandwidth.
+template <int U>
+__global__ void __launch_bounds__(KB, U > 2 ? 4 : 8) k_mgs_step(int n, const double* __restrict__ part_in, int nparts,
                                                     double* __restrict__ hout, double* __restrict__ w,
                                                     const double* __restrict__ vi, const double* __restrict__ vnext,
                                                     double* __restrict__ part_out) {
-  const double h = sum_parts(part_in, nparts);
-  if (blockIdx.x == 0 && threadIdx.x == 0 && hout) *hout = h;
   const unsigned N = (unsigned)n, S = gridDim.x * KB;
   unsigned i = blockIdx.x * KB + threadIdx.x;
+  double w0[U], v0[U], u0[U];
+  auto load = [&]() {
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      const bool in = i + (unsigned)k * S < N;
+      w0[k] = in ? w[i + (unsigned)k * S] : 0.0;
+      v0[k] = in ? vi[i + (unsigned)k * S] : 0.0;
+      u0[k] = in && vnext ? vnext[i + (unsigned)k * S] : 0.0;  // none: the partial sums of ||w||^2
+    }
+  };
+  if constexpr (U > 2) load();
+  const double h = sum_parts(part_in, nparts);
+  if (blockIdx.x == 0 && threadIdx.x == 0 && hout) *hout = h;
+  if constexpr (U <= 2) load();
   double acc = 0.0;
-  if (vnext) {
-    for (; i + S < N; i += 2 * S) {
-      const double w0 = w[i], w1 = w[i + S];
-      const double v0 = vi[i], v1 = vi[i + S];
-      const double u0 = vnext[i], u1 = vnext[i + S];
-      const double n0 = w0 - h * v0, n1 = w1 - h * v1;
-      w[i] = n0;
-      w[i + S] = n1;
-      acc += n0 * u0;
-      acc += n1 * u1;
-    }
-    for (; i < N; i += S) {
-      const double wn = w[i] - h * vi[i];
-      w[i] = wn;
-      acc += wn * vnext[i];
-    }
-  } else {  // last step: the partial sums of ||w||^2 for the normalisation
-    for (; i + S < N; i += 2 * S) {
-      const double w0 = w[i], w1 = w[i + S];
-      const double v0 = vi[i], v1 = vi[i + S];
-      const double n0 = w0 - h * v0, n1 = w1 - h * v1;
-      w[i] = n0;
-      w[i + S] = n1;
-      acc += n0 * n0;
-      acc += n1 * n1;
-    }
-    for (; i < N; i += S) {
-      const double wn = w[i] - h * vi[i];
-      w[i] = wn;
-      acc += wn * wn;
-    }
+  while (i < N) {
+#pragma unroll
+    for (int k = 0; k < U; ++k)
+      if (i + (unsigned)k * S < N) {
+        const double wn = w0[k] - h * v0[k];
+        w[i + (unsigned)k * S] = wn;
+        acc += wn * (vnext ? u0[k] : wn);
+      }
+    i += U * S;
+    if (i < N) load();
   }
   const double s = block_sum(acc);
   if (threadIdx.x == 0) part_out[blockIdx.x] = s;
@@ -121,14 +118,15 @@ __global__ void __launch_bounds__(KB, 8) k_normalize(int n, const double* __rest
   const double h = sqrt(sum_parts(part_in, nparts));
   if (blockIdx.x == 0 && threadIdx.x == 0 && hout) *hout = h;
   if (h == 0.0) return;
+  const Divider by(h);
   const unsigned N = (unsigned)n, S = gridDim.x * KB;
   unsigned i = blockIdx.x * KB + threadIdx.x;
   for (; i + S < N; i += 2 * S) {  // w may be vout: each element is read, then written, by one thread
     const double w0 = w[i], w1 = w[i + S];
-    vout[i] = w0 / h;
-    vout[i + S] = w1 / h;
+    vout[i] = by(w0);
+    vout[i + S] = by(w1);
   }
-  for (; i < N; i += S) vout[i] = w[i] / h;
+  for (; i < N; i += S) vout[i] = by(w[i]);
 }
 
 // The end of Arnoldi step j: h_{j+1,j} and v_{j+1} as k_normalize, and, by one
@@ -156,14 +154,15 @@ __global__ void __launch_bounds__(KB, 8) k_normalize_givens(int n, const double*
   }
   const double h = sqrt(sum_parts(part_in, nparts));
   if (h != 0.0) {
+    const Divider by(h);
     const unsigned N = (unsigned)n, S = gridDim.x * KB;
     unsigned i = blockIdx.x * KB + threadIdx.x;
     for (; i + S < N; i += 2 * S) {
       const double w0 = w[i], w1 = w[i + S];
-      vout[i] = w0 / h;
-      vout[i + S] = w1 / h;
+      vout[i] = by(w0);
+      vout[i + S] = by(w1);
     }
-    for (; i < N; i += S) vout[i] = w[i] / h;
+    for (; i < N; i += S) vout[i] = by(w[i]);
   }
   if (!lead || threadIdx.x != 0) return;
   for (int i = 0; i < j; ++i) {
@@ -242,9 +241,12 @@ cudaError_t launch_dot_part(int n, const double* a, const double* b, double* par
 }
 
 cudaError_t launch_mgs_step(int n, const double* part_in, double* hout, double* w, const double* vi,
-                            const double* vnext, double* part_out, cudaStream_t s) {
+                            const double* vnext, double* part_out, int sms, cudaStream_t s) {
   const int np = krylov_parts(n);
-  k_mgs_step<<<np, KB, 0, s>>>(n, part_in, np, hout, w, vi, vnext, part_out);
+  if (np <= 4 * sms)
+    k_mgs_step<4><<<np, KB, 0, s>>>(n, part_in, np, hout, w, vi, vnext, part_out);
+  else
+    k_mgs_step<2><<<np, KB, 0, s>>>(n, part_in, np, hout, w, vi, vnext, part_out);
   return cudaGetLastError();
 }
 

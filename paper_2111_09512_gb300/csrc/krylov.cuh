@@ -15,7 +15,7 @@ int krylov_parts(int n);
 cudaError_t launch_dot_part(int n, const double* a, const double* b, double* part, cudaStream_t s);
 // h = sum(part_in); if hout: *hout = h; w -= h vi; part_out = partials of w.vnext (or |w|^2 if vnext null)
 cudaError_t launch_mgs_step(int n, const double* part_in, double* hout, double* w, const double* vi,
-                            const double* vnext, double* part_out, cudaStream_t s);
+                            const double* vnext, double* part_out, int sms, cudaStream_t s);
 // h = sqrt(sum(part_in)); *hout = h; vout = w / h (skipped if h == 0)
 cudaError_t launch_normalize(int n, const double* part_in, double* hout, const double* w, double* vout,
                              cudaStream_t s);
