@@ -334,6 +334,7 @@ struct silu_batch_s {
   std::vector<InnerGraph> graphs;
   double graph_tol = -1.0;  // tol and maxit the captured iterations were made with
   int graph_maxit = -1;
+  int graph_restart = -1;  // and restart length, the leading dimension of H
   ~silu_batch_s() {
     for (InnerGraph& ig : graphs)
       if (ig.exec) cudaGraphExecDestroy(ig.exec);
@@ -646,13 +647,14 @@ silu_status silu_batch_fgmres(silu_batch B, double* x, const double* b, double t
     CK(ensure_vectors(F, 1));
     CK(ensure_bkrylov(B, m));
 
-    // captured iterations carry tol and maxit as kernel arguments
-    if (tol != B->graph_tol || maxit != B->graph_maxit) {
+    // captured iterations carry tol, maxit and the restart length as kernel arguments
+    if (tol != B->graph_tol || maxit != B->graph_maxit || m != B->graph_restart) {
       for (InnerGraph& ig : B->graphs)
         if (ig.exec) cudaGraphExecDestroy(ig.exec);
       B->graphs.clear();
       B->graph_tol = tol;
       B->graph_maxit = maxit;
+      B->graph_restart = m;
     }
     const int grid = grid_for(B);
     const int4* ch = B->d_chunks.as<int4>();

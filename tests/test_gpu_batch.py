@@ -128,3 +128,18 @@ def test_autotune_tries_sorted_copies_where_they_pay(silu, ctx):
     silu.ilu_smooth(F, x2, b, 4, 4)
     ctx.check()
     assert relerr(x2.cpu().numpy(), x1.cpu().numpy()) < 1e-12
+
+
+def test_batch_fgmres_captures_again_for_another_restart_length(silu, ctx):
+    """Captured iterations carry the leading dimension of the Hessenberg
+    matrices: a shorter restart on the same batch gives what a new batch gives."""
+    systems = systems_for([9, 14, 11], 700)
+    out = []
+    for lengths in ((8,), (20, 8)):
+        B = silu.Batch(ctx, systems, "ilu0")
+        b = torch.from_numpy(synth.rhs(B.n, 1, seed=4)[:, 0]).cuda()
+        for m in lengths:
+            x = torch.zeros(B.n, dtype=torch.float64, device="cuda")
+            r = silu.silu_batch_fgmres(B, x, b, tol=1e-9, restart=m, maxit=200)
+        out.append((x, r))
+    assert torch.equal(out[0][0], out[1][0]) and np.array_equal(out[0][1][1], out[1][1][1])
