@@ -643,10 +643,20 @@ silu_status silu_batch_fgmres(silu_batch B, double* x, const double* b, double t
   cudaStream_t s = ctx->stream;
   silu_ilu F = B->F;
   int remaining = 0;
+  int cycles = 0;  // restart cycles run: no system has more than cycles * m + j iterations
+  struct Events {
+    cudaEvent_t e[2] = {nullptr, nullptr};
+    ~Events() {
+      for (cudaEvent_t v : e)
+        if (v) cudaEventDestroy(v);
+    }
+    cudaEvent_t& operator[](int k) { return e[k]; }
+  } it_done;
   try {
     CK(ensure_vectors(F, 1));
     CK(ensure_bkrylov(B, m));
-
+    CK(cudaEventCreateWithFlags(&it_done[0], cudaEventDisableTiming));
+    CK(cudaEventCreateWithFlags(&it_done[1], cudaEventDisableTiming));
     // captured iterations carry tol, maxit and the restart length as kernel arguments
     if (tol != B->graph_tol || maxit != B->graph_maxit || m != B->graph_restart) {
       for (InnerGraph& ig : B->graphs)
@@ -686,12 +696,23 @@ silu_status silu_batch_fgmres(silu_batch B, double* x, const double* b, double t
              (k_bdivide<<<grid, KB, 0, s>>>(B->nch, ch, B->beta.as<double>(), B->act.as<int>(), V, V),
               cudaGetLastError()));
       CK(cudaMemsetAsync(B->H.p, 0, B->H.bytes, s));
-      for (int j = 0; j < m; ++j) {
+      // One iteration ahead of the host's stopping test: iteration j + 1 is
+      // queued before the count of systems still active after iteration j is
+      // read (while maxit cannot have stopped them all).  Queued past the end
+      // it finds no system active and touches nothing the update of x reads.
+      auto queue_inner = [&](int j) {
         run_inner(B, j, m, sweeps_L, sweeps_U, precond, tol, maxit);
-        CK(cudaMemcpyAsync(hp + 1, B->counter.as<int>() + 1, sizeof(int), cudaMemcpyDeviceToHost, s));
-        CK(cudaStreamSynchronize(s));
-        if (hp[1] == 0) break;
+        CK(cudaMemcpyAsync(hp + 1 + (j & 1), B->counter.as<int>() + 1, sizeof(int), cudaMemcpyDeviceToHost, s));
+        CK(cudaEventRecord(it_done[j & 1], s));
+      };
+      queue_inner(0);
+      for (int j = 0, queued = 0; j < m; ++j) {
+        if (queued == j && j + 1 < m && (long long)cycles * m + j + 1 < maxit) queue_inner(++queued);
+        CK(cudaEventSynchronize(it_done[j & 1]));
+        if (hp[1 + (j & 1)] == 0) break;
+        if (queued == j && j + 1 < m) queue_inner(++queued);
       }
+      ++cycles;
       LAUNCH(ctx, SILU_K_KRYLOV,
              (k_bupdate<<<grid, KB, sizeof(double) * (size_t)m, s>>>(B->nch, ch, B->jend.as<int>(),
                                                                      B->H.as<double>(), B->g.as<double>(), m,
