@@ -335,10 +335,11 @@ silu_status silu_ilu_set_direct(silu_ilu F, int mode);
  * residual, the sweeps on L_s and on the scaled upper factor and the update
  * of x -- in one cooperative launch whose steps are separated by grid-wide
  * barriers, instead of one launch per sweep.  Same step sequence, same
- * per-row summation order.  mode 0 (default): fused for 2 or 4 columns of
- * systems of at most 131072 rows, where launches dominate (one column runs
- * as fast through the staged sweeps, each launched as a programmatic
- * dependent of the one before); 1 never; 2 always.  Every barrier
+ * per-row summation order.  mode 0 (default): where it is the faster
+ * way, 2 or 4 columns of FP64 systems of 38913 to 131072 rows (below, and in
+ * FP32, sweeps on sliced copies, each launched as a programmatic dependent of
+ * the one before, take two thirds of the time) and systems of up to 131072
+ * rows without sliced copies; 1 never; 2 always.  Every barrier
  * wait is bounded (2 s); one that gives up makes the next silu_ctx_check
  * return SILU_ERR_TIMEOUT.  Other modes -> SILU_ERR_INVALID_ARG.
  */

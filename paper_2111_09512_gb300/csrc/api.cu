@@ -475,6 +475,13 @@ bool multi_tiles(silu_ilu F, const DevCsr& T, int R) {
   return F->variant != 1 && silu::staged_multi_ok(T, R) && (F->variant >= 2 || T.ntiles >= F->ctx->env.sms * 16);
 }
 
+// Two or four columns of a small system with row-scaled factors, in the
+// automatic mode: launches dominate.  The fused launch or the small sliced
+// kernels (use_fused); both sum every row in column order.
+bool small_block(silu_ilu F, int R) {
+  return F->fused_mode == 0 && scaled_upper(F) && (R == 2 || R == 4) && F->F.L.n <= kFusedMaxRows;
+}
+
 // Whether a launch on T takes the sliced copy: the default wherever there is
 // one.  An explicit staged shape of A (silu_mat_set_shape) and, for the
 // factors, an explicit staged variant (2, 3) keep the tiles; variant 1 keeps
@@ -482,10 +489,10 @@ bool multi_tiles(silu_ilu F, const DevCsr& T, int R) {
 bool use_slices(silu_ilu F, const DevCsr& T, int R, int ldx) {
   if (!T.sl || T.explicit_shape || F->variant == 1 || R > 4 || (R == 1 && ldx != 1)) return false;
   if (F->variant != 0 && (&T == &F->dL || &T == &F->dU)) return false;
-  // several columns of an FP32 smoother: only where the tiled multi-column
-  // sweep, which sums in the same order, would run (an FP32 sum in another
-  // order differs by 1e-7)
-  if (R > 1 && F->prec == SILU_FP32) return multi_tiles(F, T, R);
+  // several columns of an FP32 smoother: only where a kernel that sums in the
+  // same order (the tiled multi-column sweep, the fused launch) would run
+  // instead: an FP32 sum in another order differs by 1e-7
+  if (R > 1 && F->prec == SILU_FP32) return multi_tiles(F, T, R) || small_block(F, R);
   return true;
 }
 
@@ -516,12 +523,20 @@ cudaError_t sweep_launch(silu_ilu F, const DevCsr& T, silu::Mode mode, int R, in
 // ---------------------------------------------------------------------------
 // Whether one application of R columns runs as one fused cooperative launch:
 // row-scaled factors (row or row/column scaling), R = 1, 2 or 4, and, in the
-// automatic mode, several columns of a system small enough that launches
-// dominate (with one column the staged sweeps, each launched as a
-// programmatic dependent of the one before, are as fast on small systems).
-bool use_fused(silu_ilu F, int R) {
+// automatic mode, several columns of a small system where that is the faster
+// way: without sliced copies, and for FP64 beyond eight slices per SM (38912
+// rows).  5+5 applications, 7-point ILU(0), 2 / 4 columns, fused against
+// sliced sweeps: 32^3 33.5/40.9 and 21.7/28.5 us (with fill 47/66 and 32/46,
+// 27-point 51/74 and 40/59), 42^3 39/50 and 37/55 (58/86 and 59/93, 70/106 and
+// 77/121); FP32 36/38 and 19/22, at 42^3 41/46 and 31/38, at 50^3 47/61 and
+// 30/39.  (A grid-wide barrier costs 2 us; a sliced sweep launched behind its
+// predecessor's last wave 1.8 us.)
+bool use_fused(silu_ilu F, int R, int ldx) {
   if (F->fused_mode == 1 || !scaled_upper(F) || (R != 1 && R != 2 && R != 4)) return false;
-  return F->fused_mode == 2 || (R > 1 && F->F.L.n <= kFusedMaxRows);
+  if (F->fused_mode == 2) return true;
+  if (!small_block(F, R)) return false;
+  const bool sliced = use_slices(F, F->A->d, R, ldx) && use_slices(F, F->dL, R, ldx) && use_slices(F, F->dU, R, ldx);
+  return !sliced || (F->prec != SILU_FP32 && F->A->d.sl->ns > 8 * F->ctx->env.sms);
 }
 
 void smooth_chunk(silu_ilu F, double* x, const double* b, int R, int ldx, size_t col, int mL, int mU, bool x_zero) {
@@ -536,7 +551,7 @@ void smooth_chunk(silu_ilu F, double* x, const double* b, int R, int ldx, size_t
   char* bufC = F->ws.c.as<char>() + col * es;
   char* bufP0 = F->ws.p0.as<char>() + col * es;
   char* bufP1 = F->ws.p1.as<char>() + col * es;
-  if (use_fused(F, R)) {
+  if (use_fused(F, R, ldx)) {
     const bool rc = F->scale == SILU_SCALE_ROWCOL;
     LAUNCH(F->ctx, SILU_K_FUSED,
            silu::launch_smooth_fused(A, F->dL, F->dU, f32, R, ldx, mL, mU, x_zero, rc, dinv,

@@ -109,6 +109,39 @@ cudaError_t fill(const DevCsr& d, const Slices& S, cudaStream_t s) {
 template <class VO, class CT, int LN>
 using Double1 = SliceKernel<double, double, VO, CT, 1, LN == 4 ? 2 : 1, LN == 4 ? 4 : 6, false, LN>;
 
+// The same for small matrices of 16-bit columns: a whole row per chunk where
+// the registers of one block per SM (two beyond eight slices per SM) allow.
+template <class VO, int LN, int CP, int MINB>
+using DoubleSmall = SliceKernel<double, double, VO, uint16_t, 1, CP, MINB, false, LN>;
+
+template <class VO>
+cudaError_t double1_small(const DevCsr& T, const LaunchEnv& env, const void* c, const void* in, void* out,
+                          const double* dinv, double* x, int epi, cudaStream_t s) {
+  const int w = T.sl->widest;
+  const bool one = T.sl->ns <= kSliceThreads / 32 * env.sms;  // one block per SM
+  auto go = [&](auto k) { return decltype(k)::launch(T, env, 1, c, in, out, dinv, x, epi, s); };
+  switch (T.sl->lanes) {
+    case 1:
+      if (w <= 4) return go(DoubleSmall<VO, 1, 2, 2>());
+      return w <= 10 || !one ? go(DoubleSmall<VO, 1, 5, 2>()) : go(DoubleSmall<VO, 1, 7, 1>());
+    case 2: return one ? go(DoubleSmall<VO, 2, 7, 1>()) : go(DoubleSmall<VO, 2, 5, 2>());
+    case 4: return one ? go(DoubleSmall<VO, 4, 8, 1>()) : go(DoubleSmall<VO, 4, 4, 2>());
+  }
+  return cudaErrorInvalidValue;
+}
+
+template <class F, class VO>
+cudaError_t each_small(F f) {
+  cudaError_t e = f(DoubleSmall<VO, 1, 2, 2>());
+  if (e == cudaSuccess) e = f(DoubleSmall<VO, 1, 5, 2>());
+  if (e == cudaSuccess) e = f(DoubleSmall<VO, 1, 7, 1>());
+  if (e == cudaSuccess) e = f(DoubleSmall<VO, 2, 7, 1>());
+  if (e == cudaSuccess) e = f(DoubleSmall<VO, 2, 5, 2>());
+  if (e == cudaSuccess) e = f(DoubleSmall<VO, 4, 8, 1>());
+  if (e == cudaSuccess) e = f(DoubleSmall<VO, 4, 4, 2>());
+  return e;
+}
+
 template <class VO, class CT>
 cudaError_t double1(const DevCsr& T, const LaunchEnv& env, const void* c, const void* in, void* out,
                     const double* dinv, double* x, int epi, cudaStream_t s) {
@@ -139,6 +172,8 @@ cudaError_t for_each_shape(F f) {
   add(f(Double1<float, int, 1>()));
   add(f(Double1<float, int, 2>()));
   add(f(Double1<float, int, 4>()));
+  add(each_small<F, double>(f));
+  add(each_small<F, float>(f));
   add(f(SliceKernel<float, float, float, uint16_t, 1, 2, 6, false>()));
   add(f(SliceKernel<float, float, float, uint16_t, 1, 4, 3, false>()));
   add(f(SliceKernel<float, float, float, uint16_t, 1, 7, 3, false>()));
@@ -225,19 +260,22 @@ cudaError_t launch_sweep_slices(const DevCsr& T, Mode mode, const LaunchEnv& env
   if (R > 1) return launch_slices_multi(T, mode, env, R, ldx, c, in, out, dinv, x, epi, s);
   if (slices_ring_fits(T, mode, env.sms)) return launch_slices_ring(T, env, c, in, out, dinv, x, epi, s);
   const bool wide = T.sl->wide;
+  const bool small = !wide && slice_small(T.sl->ns, env.sms);
   // FP32, which only small matrices reach: a whole row per chunk where rows
   // allow (27-point 32^3 4.5 us a sweep).
   const double mean = (double)T.sl->slots / (32.0 * (double)T.sl->ns);
   auto go = [&](auto k) { return decltype(k)::launch(T, env, ldx, c, in, out, dinv, x, epi, s); };
   switch (mode) {
     case MODE_D:
+      if (small) return double1_small<double>(T, env, c, in, out, dinv, x, epi, s);
       return wide ? double1<double, int>(T, env, c, in, out, dinv, x, epi, s)
                   : double1<double, uint16_t>(T, env, c, in, out, dinv, x, epi, s);
     case MODE_DF:
+      if (small) return double1_small<float>(T, env, c, in, out, dinv, x, epi, s);
       return wide ? double1<float, int>(T, env, c, in, out, dinv, x, epi, s)
                   : double1<float, uint16_t>(T, env, c, in, out, dinv, x, epi, s);
     case MODE_F:
-      if (mean <= 4.0)
+      if (mean <= 4.0 && !(small && T.sl->widest > 4))
         return wide ? go(SliceKernel<float, float, float, int, 1, 2, 5, false>())
                     : go(SliceKernel<float, float, float, uint16_t, 1, 2, 6, false>());
       if (wide || mean <= 8.0 || mean > 14.0)

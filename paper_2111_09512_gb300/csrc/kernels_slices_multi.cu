@@ -3,6 +3,8 @@
 // it; two to four entries per chunk keep R columns of gathers in registers.
 #include "slices.cuh"
 
+#include <type_traits>
+
 namespace silu {
 namespace {
 
@@ -15,6 +17,27 @@ struct MultiShape {
 
 template <class MT, class VI, class VO, class CT, int R, bool VEC>
 using MultiKernel = SliceKernel<MT, VI, VO, CT, R, MultiShape<MT, R>::CP, MultiShape<MT, R>::MINB, VEC>;
+
+// Small matrices (16-bit columns): rows of up to 4 entries in one chunk, longer
+// ones 8 at a time.
+template <class MT, class VI, class VO, int R, bool VEC, int CP>
+using SmallKernel = SliceKernel<MT, VI, VO, uint16_t, R, CP, 1, VEC>;
+
+template <class MT, class VI, class VO, int R, bool VEC>
+cudaError_t prepare_small() {
+  const cudaError_t e = SmallKernel<MT, VI, VO, R, VEC, 2>::prepare();
+  return e == cudaSuccess ? SmallKernel<MT, VI, VO, R, VEC, 4>::prepare() : e;
+}
+
+template <class MT, class VI, class VO>
+cudaError_t prepare_small_mode() {
+  cudaError_t e = prepare_small<MT, VI, VO, 2, false>();
+  if (e == cudaSuccess) e = prepare_small<MT, VI, VO, 2, true>();
+  if (e == cudaSuccess) e = prepare_small<MT, VI, VO, 3, false>();
+  if (e == cudaSuccess) e = prepare_small<MT, VI, VO, 4, false>();
+  if (e == cudaSuccess) e = prepare_small<MT, VI, VO, 4, true>();
+  return e;
+}
 
 template <class MT, class VI, class VO, class CT>
 cudaError_t prepare_mode() {
@@ -35,6 +58,25 @@ cudaError_t multi(const DevCsr& T, const LaunchEnv& env, int R, int ldx, const v
   const bool vec = R != 3 && ldx % (int)(unit / sizeof(VI)) == 0 && (uintptr_t)in % unit == 0 &&
                    (uintptr_t)c % unit == 0;
   auto go = [&](auto k) { return decltype(k)::launch(T, env, ldx, c, in, out, dinv, x, epi, s); };
+  if constexpr (sizeof(CT) == 2) {
+    if (slice_small(T.sl->ns, env.sms)) {
+      auto pick = [&](auto r, auto v) {
+        constexpr int RR = decltype(r)::value;
+        constexpr bool VV = decltype(v)::value;
+        return T.sl->widest <= 4 ? go(SmallKernel<MT, VI, VO, RR, VV, 2>()) : go(SmallKernel<MT, VI, VO, RR, VV, 4>());
+      };
+      using std::integral_constant;
+      switch (R) {
+        case 2:
+          return vec ? pick(integral_constant<int, 2>(), std::true_type())
+                     : pick(integral_constant<int, 2>(), std::false_type());
+        case 3: return pick(integral_constant<int, 3>(), std::false_type());
+        case 4:
+          return vec ? pick(integral_constant<int, 4>(), std::true_type())
+                     : pick(integral_constant<int, 4>(), std::false_type());
+      }
+    }
+  }
   switch (R) {
     case 2: return vec ? go(MultiKernel<MT, VI, VO, CT, 2, true>()) : go(MultiKernel<MT, VI, VO, CT, 2, false>());
     case 3: return go(MultiKernel<MT, VI, VO, CT, 3, false>());
@@ -63,6 +105,9 @@ cudaError_t slices_prepare_multi() {
   if (e == cudaSuccess) e = prepare_mode<float, float, float, int>();
   if (e == cudaSuccess) e = prepare_mode<double, double, float, uint16_t>();
   if (e == cudaSuccess) e = prepare_mode<double, double, float, int>();
+  if (e == cudaSuccess) e = prepare_small_mode<double, double, double>();
+  if (e == cudaSuccess) e = prepare_small_mode<float, float, float>();
+  if (e == cudaSuccess) e = prepare_small_mode<double, double, float>();
   return e;
 }
 

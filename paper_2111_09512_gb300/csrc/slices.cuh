@@ -20,9 +20,16 @@
 // Each lane accumulates c_i - sum t_ij in_j in column order with one FMA per
 // entry, in LN partial sums for rows that the tiled sweep gives to LN lanes
 // (entry k into sum k mod LN, then the sums added as that sweep's lanes add
-// theirs), so results are the tiled sweep's bits; a padded entry multiplies 0 by 0, which leaves the accumulator as it
-// is (its column is not read, so an infinite or NaN entry of `in` reaches only
-// the rows that refer to it).
+// theirs), so results are the tiled sweep's bits; a padded entry multiplies 0 by 0,
+// which leaves the accumulator as it is (its column is not read, so an
+// infinite or NaN entry of `in` reaches only the rows that refer to it).
+//
+// The next launch is released (its blocks become resident and read their
+// first entries) only once this one may start: were it released at once, the
+// blocks of three and more later launches would fill the SMs, and a launch
+// would start wherever room happened to be left, two blocks on some SMs and
+// none on others (24^3 ILUT 5+5 application 24.2 -> 19 us, 42^3 ILUT 10+10
+// 62.8 -> 59.5 us, 128^3 823 -> 819 us).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -132,24 +139,33 @@ constexpr unsigned kEpiDinv = 1u << EPI_SCALE | 1u << EPI_SCALE_ADDX | 1u << EPI
                               1u << EPI_JAC_ADDX | 1u << EPI_JAC_SETX;
 constexpr unsigned kEpiX = 1u << EPI_ADDX | 1u << EPI_SCALE_ADDX | 1u << EPI_JAC_ADDX | 1u << EPI_RICH_ADDX;
 
-// CP pairs of entries per chunk, at least MINB blocks of 8 warps per SM, LN
-// partial sums per row.
+// Launch flag of small matrices, beside the L2 flags: block b of B walks the
+// slices [b ns / B, (b + 1) ns / B) (ns and B are small) instead of every
+// (B W)-th group of W.
+constexpr int kFlagSpread = 8;
+
+// CP pairs of entries per chunk, at least MINB blocks of (up to) 8 warps per SM,
+// LN partial sums per row.
 template <class MT, class VI, class VO, class CT, int R, int CP, int MINB, bool VEC, int LN>
 __global__ void __launch_bounds__(kSliceThreads, MINB)
     k_slices(int ns, int n, const int2* __restrict__ hdr, const CT* __restrict__ ci, const MT* __restrict__ va,
              const VI* __restrict__ c, const VI* __restrict__ in, VO* __restrict__ out, int ldx,
              const double* __restrict__ dinv, double* __restrict__ x, int epi, int flags) {
   static_assert(2 * CP % LN == 0, "a chunk starts at the first partial sum");
-  constexpr int W = kSliceThreads / 32;
+  const int W = blockDim.x >> 5;
   const int ld = R == 1 ? 1 : ldx;
   const int lane = threadIdx.x & 31;
-  const int nw = gridDim.x * W;
-  int s = blockIdx.x * W + (threadIdx.x >> 5);
+  const bool spread = (flags & kFlagSpread) != 0;
+  const int nw = spread ? W : gridDim.x * W;
+  int s = blockIdx.x * W + (threadIdx.x >> 5), end = ns;
+  if (spread) {
+    s = (int)((unsigned)blockIdx.x * (unsigned)ns / gridDim.x) + (threadIdx.x >> 5);
+    end = (int)(((unsigned)blockIdx.x + 1u) * (unsigned)ns / gridDim.x);
+  }
   const bool rev = (flags & kFlagReverse) != 0;
   const uint64_t stream = (flags & kFlagFactorNormal) ? policy_evict_normal() : policy_evict_first();
   const uint64_t keep = (flags & kFlagVectorNormal) ? policy_evict_normal() : policy_evict_last();
-  grid_launch_dependents();
-  if (s >= ns) {
+  if (s >= end) {
     grid_wait_prior();
     return;
   }
@@ -191,12 +207,13 @@ __global__ void __launch_bounds__(kSliceThreads, MINB)
   s += nw;
   int nsl = 0, npe = 0;
   int2 nh = make_int2(0, 0);
-  if (s < ns) {
+  if (s < end) {
     nsl = rev ? ns - 1 - s : s;
     nh = __ldg(hdr + nsl);
     npe = __ldg(&hdr[nsl + 1].x);
   }
   grid_wait_prior();  // c, in, out and x below belong to the previous kernel until it completes
+  grid_launch_dependents();
   int row = sl * 32 + lane;
   MT acc[LN][R];  // acc[0] starts at c
   auto clear_rest = [&]() {
@@ -231,7 +248,7 @@ __global__ void __launch_bounds__(kSliceThreads, MINB)
     if (!last) {
       load(p, pe);
     } else {
-      more = s < ns;
+      more = s < end;
       if (more) {
         h = nh;
         p = h.x;
@@ -240,7 +257,7 @@ __global__ void __launch_bounds__(kSliceThreads, MINB)
         load(p, pe);
         start_row(row, nacc);
         s += nw;
-        if (s < ns) {
+        if (s < end) {
           nsl = rev ? ns - 1 - s : s;
           nh = __ldg(hdr + nsl);
           npe = __ldg(&hdr[nsl + 1].x);
@@ -279,6 +296,28 @@ __global__ void __launch_bounds__(kSliceThreads, MINB)
   }
 }
 
+// Matrices of at most 16 slices per SM: a launch is a chain of latencies, so a
+// chunk takes a whole row (one round of gathers), whatever registers it needs,
+// and the slices are split evenly over one block per SM (two beyond eight
+// slices per SM), each of no more warps than its share.  (Blocks of eight
+// warps leave SMs idle while the four FP64 partitions of others queue.)
+constexpr int kSliceSmall = 16;
+inline bool slice_small(int ns, int sms) { return ns <= kSliceSmall * sms; }
+
+struct SlicePlan {
+  int warps, blocks, flags;
+};
+inline SlicePlan slice_plan(int ns, int sms, int most) {
+  constexpr int W = kSliceThreads / 32;
+  if (!slice_small(ns, sms)) {
+    const int want = (ns + W - 1) / W;
+    return {W, want < sms * most ? want : sms * most, 0};
+  }
+  const int full = ns > W * sms && most > 1 ? 2 * sms : sms;
+  const int blocks = ns < full ? ns : full, share = (ns + blocks - 1) / blocks;
+  return {share < W ? share : W, blocks, kFlagSpread};
+}
+
 template <class MT, class VI, class VO, class CT, int R, int CP, int MINB, bool VEC, int LN = 1>
 struct SliceKernel {
   static cudaError_t prepare() {
@@ -290,12 +329,10 @@ struct SliceKernel {
                             const double* dinv, double* x, int epi, cudaStream_t s) {
     const Slices& S = *T.sl;
     if (S.ns == 0) return cudaSuccess;
-    constexpr int W = kSliceThreads / 32;
-    const int want = (S.ns + W - 1) / W;
-    const int most = env.sms * MINB;
+    const SlicePlan plan = slice_plan(S.ns, env.sms, MINB);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(want < most ? want : most));
-    cfg.blockDim = dim3(kSliceThreads);
+    cfg.gridDim = dim3((unsigned)plan.blocks);
+    cfg.blockDim = dim3((unsigned)(plan.warps * 32));
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -304,7 +341,7 @@ struct SliceKernel {
     cfg.numAttrs = env.overlap ? 1 : 0;
     // consecutive launches alternate their direction, so each starts on the
     // rows that the previous one touched last, while they are still in L2
-    int flags = env.l2 & (kFlagFactorNormal | kFlagVectorNormal);
+    int flags = plan.flags | (env.l2 & (kFlagFactorNormal | kFlagVectorNormal));
     if ((env.l2 & kFlagReverse) && (env.flips++ & 1u)) flags |= kFlagReverse;
     return cudaLaunchKernelEx(&cfg, k_slices<MT, VI, VO, CT, R, CP, MINB, VEC, LN>, S.ns, T.n, (const int2*)S.hdr,
                               (const CT*)S.ci, (const MT*)S.va, (const VI*)c, (const VI*)in, (VO*)out, ldx, dinv, x,

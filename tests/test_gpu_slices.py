@@ -149,3 +149,34 @@ def test_refactor_renews_the_slices_of_the_matrix(silu, ctx):
     r = dev(np.zeros((n, 1)))
     M.residual(r, dev(x0), dev(b))
     assert relerr(host(r), oracle.residual(A2, x0, b)) < FP64_TOL
+
+
+# one, one and a bit, eight and a bit, sixteen and sixteen and a bit slices of 32 rows per SM of 152
+SMALL = [pytest.param(size, gen, kind, id=f"{gen}-{kind}-{'x'.join(map(str, size))}")
+         for size in ((12, 11, 13), (17, 16, 18), (34, 34, 34), (43, 43, 42), (43, 43, 44))
+         for gen, kind in (("cutcell7", "ilu0"), ("cutcell7", "ilut"), ("hex27", "ilu0"))]
+
+
+@pytest.mark.parametrize("size,gen,kind", SMALL)
+def test_small_systems_match_the_lanes_per_row_kernel(silu, ctx, size, gen, kind):
+    """Automatic choice (small sliced kernels or the fused launch) against the general kernel: sums of
+    at most 28 terms of a scaled system, eight sweeps, so rounding of order 1e-14 (FP32 1e-5)."""
+    A = getattr(synth, gen)(*size, seed=6)
+    n = len(A[0]) - 1
+    M = silu.Matrix(ctx, *A)
+    for scale in (silu.SCALE_ROW, silu.SCALE_ROWCOL):
+        for prec, tol in ((silu.FP64, FP64_TOL), (silu.FP32, 1e-5)):
+            F = silu.ilu_setup(ctx, M, kind, 1e-3, 10, scale=scale, prec=prec)
+            for nrhs in (1, 2, 3, 4):
+                b, x0 = synth.rhs(n, nrhs, seed=7), synth.rhs(n, nrhs, seed=8)
+                out = []
+                for variant, fused in ((0, 0), (1, 1), (0, 2)):
+                    F.set_kernel(variant)
+                    F.set_fused(fused)
+                    x = dev(x0)
+                    silu.ilu_smooth(F, x, dev(b), 5, 4)
+                    ctx.check()
+                    out.append(host(x))
+                assert max(relerr(out[0][:, k], out[1][:, k]) for k in range(nrhs)) < tol, (scale, prec, nrhs)
+                if prec == silu.FP32 and nrhs in (2, 4):  # the fused launch's order of summation
+                    assert np.array_equal(out[0], out[2]), (scale, nrhs)
