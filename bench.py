@@ -103,7 +103,7 @@ def load_peaks():
 
 def sweep_source_hash():
     h = hashlib.sha256()
-    for f in ("kernels_staged.cu", "device.cuh"):
+    for f in ("slices.cuh", "kernels_slices.cu", "kernels_slices_ring.cu", "sweep_ptx.cuh", "device.cuh"):
         with open(os.path.join(ROOT, "paper_2111_09512_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]

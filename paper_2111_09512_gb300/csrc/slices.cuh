@@ -14,7 +14,7 @@
 // always has one chunk in flight.  Measured against the tiled CSR sweeps
 // (k_sweep_rows, k_sweep_staged, k_sweep_multi): 128^3 cut-cell ILUT FP64
 // lower / upper sweep 45.9 / 49.6 -> 43.9 / 43.9 us (20.9 M slots: 477 G/s),
-// 24^3 ILUT application 83 -> 61 us, 160^3 27-point FP64 residual 290 -> 232 us,
+// 24^3 ILUT 10+10 application 83 -> 38 us, 160^3 27-point FP64 residual 290 -> 232 us,
 // three columns of the 101 x 97 x 89 box 1111 -> 507 us per application.
 //
 // Each lane accumulates c_i - sum t_ij in_j in column order with one FMA per
@@ -299,8 +299,14 @@ __global__ void __launch_bounds__(kSliceThreads, MINB)
 // Matrices of at most 16 slices per SM: a launch is a chain of latencies, so a
 // chunk takes a whole row (one round of gathers), whatever registers it needs,
 // and the slices are split evenly over one block per SM (two beyond eight
-// slices per SM), each of no more warps than its share.  (Blocks of eight
-// warps leave SMs idle while the four FP64 partitions of others queue.)
+// slices per SM), each of no more warps than its share: blocks of eight warps
+// leave SMs idle while the four FP64 partitions of others queue (24^3 ILUT
+// 10+10 application 60 us that way, 38.3 us this way).  The line: 5+5
+// applications at 10 slices per SM (36^3), 1 / 2 / 4 columns, this way
+// against the large matrices' way: ILU(0) 27.0 / 36.3 / 52.5 and 27.7 / 46.6 /
+// 67.5 us, ILUT 34.5 / 57.4 / 89.6 and 52.7 / 78 / 111 us; at 25 slices per SM
+// (50^3), where several rounds per warp are needed either way, ILUT four
+// columns 122 us the large way.
 constexpr int kSliceSmall = 16;
 inline bool slice_small(int ns, int sms) { return ns <= kSliceSmall * sms; }
 
