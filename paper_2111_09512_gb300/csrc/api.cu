@@ -489,6 +489,18 @@ bool small_block(silu_ilu F, int R) {
 bool use_slices(silu_ilu F, const DevCsr& T, int R, int ldx) {
   if (!T.sl || T.explicit_shape || F->variant == 1 || R > 4 || (R == 1 && ldx != 1)) return false;
   if (F->variant != 0 && (&T == &F->dL || &T == &F->dU)) return false;
+  // Large matrices that the tiled sweeps serve faster (per sweep, slices
+  // against tiles):
+  // - FP32, one column, int32 columns (no fewer bytes than the tiles, and no
+  //   ring): 27-point 260 x 260 x 30 factors 45.6 / 35.4 us, x 6 8.7 / 7.5 us
+  //   (below 64 slices per SM slices win: x 2 3.6 / 3.8 us);
+  // - two columns, and four in FP64, of rows of more than ten entries (more
+  //   than a few chunks of gathers per slice): 27-point 130^3 FP64 127 / 104
+  //   and 236 / 206 us, FP32 two columns 54.7 / 43.4 us; four FP32 columns
+  //   66.9 / 82.9 us, and cut-cell 100^3 ILUT rows of ten 44.0 / 44.5 and
+  //   79.8 / 85.6 us.
+  if (R == 1 && T.fp32 && T.sl->wide && T.ntiles > 0 && T.sl->ns >= 64 * F->ctx->env.sms) return false;
+  if (R > 1 && !(T.fp32 && R == 4) && T.sl->widest > 10 && multi_tiles(F, T, R)) return false;
   // several columns of an FP32 smoother: only where a kernel that sums in the
   // same order (the tiled multi-column sweep, the fused launch) would run
   // instead: an FP32 sum in another order differs by 1e-7

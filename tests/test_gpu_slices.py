@@ -180,3 +180,25 @@ def test_small_systems_match_the_lanes_per_row_kernel(silu, ctx, size, gen, kind
                 assert max(relerr(out[0][:, k], out[1][:, k]) for k in range(nrhs)) < tol, (scale, prec, nrhs)
                 if prec == silu.FP32 and nrhs in (2, 4):  # the fused launch's order of summation
                     assert np.array_equal(out[0], out[2]), (scale, nrhs)
+
+
+@pytest.mark.parametrize("gen", [lambda: synth.hex27(46, 45, 44, seed=2), lambda: synth.hex27(262, 258, 5, seed=2)],
+                         ids=["16-bit columns", "int32 columns"])
+def test_long_rows_and_int32_columns_match_the_lanes_per_row_kernel(silu, ctx, gen):
+    """Rows of up to 13 factor entries on both sides of the lines between slices and tiles."""
+    A = gen()
+    n = len(A[0]) - 1
+    M = silu.Matrix(ctx, *A)
+    for prec, tol in ((silu.FP64, FP64_TOL), (silu.FP32, 1e-5)):
+        F = silu.ilu_setup(ctx, M, "ilu0", prec=prec)
+        for nrhs in (1, 2, 3, 4):
+            b, x0 = synth.rhs(n, nrhs, seed=9), synth.rhs(n, nrhs, seed=10)
+            out = []
+            for variant, fused in ((0, 0), (1, 1)):
+                F.set_kernel(variant)
+                F.set_fused(fused)
+                x = dev(x0)
+                silu.ilu_smooth(F, x, dev(b), 3, 4)
+                ctx.check()
+                out.append(host(x))
+            assert max(relerr(out[0][:, k], out[1][:, k]) for k in range(nrhs)) < tol, (prec, nrhs)
