@@ -30,7 +30,7 @@ struct RingStage {
 template <class MT, class VI, class VO, int G, int W, int D>
 __global__ void __launch_bounds__(W * 32, 1)
     k_slices_ring(int ns, int n, const int2* __restrict__ hdr, const uint16_t* __restrict__ ci,
-                  const MT* __restrict__ va, const VI* __restrict__ c, const VI* __restrict__ in,
+                  const MT* __restrict__ va, const VI* c, const VI* in,
                   VO* __restrict__ out, const double* __restrict__ dinv, double* __restrict__ x, int epi, int flags,
                   int* __restrict__ err) {
   using S = RingStage<MT>;

@@ -179,7 +179,7 @@ __device__ __forceinline__ void issue_tile(int4 d, unsigned char* st, uint64_t* 
 // before the first FMA; the FMA loop runs to the warp's longest row.  One
 // factor entry read from shared memory feeds R FMAs.
 template <class MT, class VI, bool NEG, int R, int CH>
-__device__ __forceinline__ void row_accumulate_cols(const MT* sv, const int* sc, int len, const VI* __restrict__ in,
+__device__ __forceinline__ void row_accumulate_cols(const MT* sv, const int* sc, int len, const VI* in,
                                                     int ldx, MT (&acc)[R], uint64_t keep) {
   const int wmax = __reduce_max_sync(0xffffffffu, len);
   for (int k0 = 0; k0 < wmax; k0 += CH) {
@@ -216,7 +216,7 @@ __device__ __forceinline__ void row_accumulate_cols(const MT* sv, const int* sc,
 // lane, plus log2(G) adds per row.
 template <class MT, class VI, bool NEG, int G, int kChunk>
 __device__ __forceinline__ MT row_accumulate(const MT* sv, const int* sc, int len, int sub,
-                                             const VI* __restrict__ in, MT acc, uint64_t keep) {
+                                             const VI* in, MT acc, uint64_t keep) {
   const int cnt = len > sub ? (len - sub + G - 1) / G : 0;  // this lane's entries
   const int wmax = __reduce_max_sync(0xffffffffu, cnt);
   for (int k0 = 0; k0 < wmax; k0 += kChunk) {
@@ -255,7 +255,7 @@ __device__ __forceinline__ MT row_accumulate(const MT* sv, const int* sc, int le
 template <class MT, class VI, class VO, int CH, int RL, bool PERM>
 __device__ __forceinline__ void rows_accumulate(const MT* sv, const int* sc, const int* sr, const int* sp, int r0,
                                                 int r1, int q0, int a0, int c0, int p0, int lane,
-                                                const VI* __restrict__ c, const VI* __restrict__ in,
+                                                const VI* c, const VI* in,
                                                 VO* __restrict__ out, const double* __restrict__ dinv,
                                                 double* __restrict__ x, int epi, uint64_t keep) {
   // entries of each row per round: CH / RL, at most 3 in FP64 (the 96
@@ -311,8 +311,8 @@ __device__ __forceinline__ void rows_accumulate(const MT* sv, const int* sc, con
 template <class MT, class VI, class VO, int G, int CH, int RL, bool PERM>
 __global__ void __launch_bounds__(warps_of<MT>() * 32, 1)
     k_sweep_staged(int ntiles, const int4* __restrict__ tiles, const int* __restrict__ rp, const int* __restrict__ ci,
-                   const MT* __restrict__ va, const int* __restrict__ perm, const VI* __restrict__ c,
-                   const VI* __restrict__ in, VO* __restrict__ out, const double* __restrict__ dinv,
+                   const MT* __restrict__ va, const int* __restrict__ perm, const VI* c,
+                   const VI* in, VO* __restrict__ out, const double* __restrict__ dinv,
                    double* __restrict__ x, int epi, int flags, int* __restrict__ err) {
   using L = StageLayout<MT, RL, PERM>;
   constexpr int kWarps = warps_of<MT>();
@@ -418,7 +418,7 @@ __global__ void __launch_bounds__(warps_of<MT>() * 32, 1)
 template <class MT, class VI, class VO, int CH, int RL, int R>
 __global__ void __launch_bounds__(warps_of<MT>() * 32, 1)
     k_sweep_multi(int ntiles, const int4* __restrict__ tiles, const int* __restrict__ rp, const int* __restrict__ ci,
-                  const MT* __restrict__ va, const VI* __restrict__ c, const VI* __restrict__ in, VO* __restrict__ out,
+                  const MT* __restrict__ va, const VI* c, const VI* in, VO* __restrict__ out,
                   int ldx, const double* __restrict__ dinv, double* __restrict__ x, int epi, int flags,
                   int* __restrict__ err) {
   using L = StageLayout<MT, RL, false>;
@@ -587,7 +587,7 @@ __device__ __forceinline__ int4 shfl_int4(int4 v, int src) {
 template <class MT, class VI, class VO, int CH, int W = warps_of<MT>(), int NNZ = kTileNnz>
 __global__ void __launch_bounds__(W * 32, 1)
     k_sweep_rows(int ntiles, const int4* __restrict__ tiles, const int* __restrict__ rp, const int* __restrict__ ci,
-                 const MT* __restrict__ va, const VI* __restrict__ c, const VI* __restrict__ in, VO* __restrict__ out,
+                 const MT* __restrict__ va, const VI* c, const VI* in, VO* __restrict__ out,
                  const double* __restrict__ dinv, double* __restrict__ x, int epi, int flags, int* __restrict__ err) {
   using L = StageLayout<MT, 1, false, NNZ>;
   constexpr int kWarps = W;

@@ -93,7 +93,7 @@ struct SliceCols<int, CP> {
   static __device__ __forceinline__ bool padded(unsigned c) { return c == 0xffffffffu; }
 };
 
-// R adjacent vector entries.  VEC: in 16-byte (or, two floats, 8-byte) loads,
+// R adjacent vector entries (ordered as ld_keep's).  VEC: in 16-byte (or, two floats, 8-byte) loads,
 // for pointers and leading dimensions that keep every row's entries aligned.
 template <class MT, int R, bool VEC>
 __device__ __forceinline__ void ld_cols(const double* p, uint64_t pol, MT (&v)[R]) {
@@ -101,7 +101,10 @@ __device__ __forceinline__ void ld_cols(const double* p, uint64_t pol, MT (&v)[R
 #pragma unroll
     for (int k = 0; k < R; k += 2) {
       double a, b;
-      asm("ld.global.nc.L2::cache_hint.v2.f64 {%0, %1}, [%2], %3;" : "=d"(a), "=d"(b) : "l"(p + k), "l"(pol));
+      asm volatile("ld.global.L2::cache_hint.v2.f64 {%0, %1}, [%2], %3;"
+                   : "=d"(a), "=d"(b)
+                   : "l"(p + k), "l"(pol)
+                   : "memory");
       v[k] = (MT)a;
       v[k + 1] = (MT)b;
     }
@@ -114,16 +117,20 @@ template <class MT, int R, bool VEC>
 __device__ __forceinline__ void ld_cols(const float* p, uint64_t pol, MT (&v)[R]) {
   if constexpr (VEC && R == 4) {
     float a, b, c, d;
-    asm("ld.global.nc.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;"
-        : "=f"(a), "=f"(b), "=f"(c), "=f"(d)
-        : "l"(p), "l"(pol));
+    asm volatile("ld.global.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;"
+                 : "=f"(a), "=f"(b), "=f"(c), "=f"(d)
+                 : "l"(p), "l"(pol)
+                 : "memory");
     v[0] = a;
     v[1] = b;
     v[2] = c;
     v[3] = d;
   } else if constexpr (VEC && R == 2) {
     float a, b;
-    asm("ld.global.nc.L2::cache_hint.v2.f32 {%0, %1}, [%2], %3;" : "=f"(a), "=f"(b) : "l"(p), "l"(pol));
+    asm volatile("ld.global.L2::cache_hint.v2.f32 {%0, %1}, [%2], %3;"
+                 : "=f"(a), "=f"(b)
+                 : "l"(p), "l"(pol)
+                 : "memory");
     v[0] = a;
     v[1] = b;
   } else {
@@ -149,7 +156,7 @@ constexpr int kFlagSpread = 8;
 template <class MT, class VI, class VO, class CT, int R, int CP, int MINB, bool VEC, int LN>
 __global__ void __launch_bounds__(kSliceThreads, MINB)
     k_slices(int ns, int n, const int2* __restrict__ hdr, const CT* __restrict__ ci, const MT* __restrict__ va,
-             const VI* __restrict__ c, const VI* __restrict__ in, VO* __restrict__ out, int ldx,
+             const VI* c, const VI* in, VO* __restrict__ out, int ldx,
              const double* __restrict__ dinv, double* __restrict__ x, int epi, int flags) {
   static_assert(2 * CP % LN == 0, "a chunk starts at the first partial sum");
   const int W = blockDim.x >> 5;

@@ -29,15 +29,18 @@ __device__ __forceinline__ uint64_t policy_evict_last() {
   return p;
 }
 
-// Vector accesses that keep the iterates resident in L2 across sweeps.
+// Vector accesses that keep the iterates resident in L2 across sweeps.  A sweep
+// may be resident while the kernel before it still writes these vectors: the
+// loads stay behind griddepcontrol.wait (volatile, memory clobber) and are
+// ordinary ones (an .nc load is for data that nobody writes meanwhile).
 __device__ __forceinline__ double ld_keep(const double* p, uint64_t pol) {
   double v;
-  asm("ld.global.nc.L2::cache_hint.f64 %0, [%1], %2;" : "=d"(v) : "l"(p), "l"(pol));
+  asm volatile("ld.global.L2::cache_hint.f64 %0, [%1], %2;" : "=d"(v) : "l"(p), "l"(pol) : "memory");
   return v;
 }
 __device__ __forceinline__ float ld_keep(const float* p, uint64_t pol) {
   float v;
-  asm("ld.global.nc.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(p), "l"(pol));
+  asm volatile("ld.global.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(p), "l"(pol) : "memory");
   return v;
 }
 __device__ __forceinline__ void st_keep(double* p, double v, uint64_t pol) {
