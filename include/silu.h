@@ -441,6 +441,15 @@ silu_status silu_ilu_set_lanes(silu_ilu F, int lanes_L, int lanes_U, int lanes_A
  * bits.
  */
 silu_status silu_ilu_set_kernel(silu_ilu F, int variant);
+/*
+ * Self-test of the bounded waits of FGMRES's one-launch Arnoldi step and of
+ * what they leave behind: a GPU thread waits (2 s) for a partial sum that
+ * nothing publishes, so that the next silu_ctx_check returns
+ * SILU_ERR_TIMEOUT, and F's exchange buffer is filled with stale entries
+ * numbered like those of a next solve, which must not take them for its own.
+ * Allocates F's FGMRES workspace if there is none.  Asynchronous.
+ */
+silu_status silu_ilu_selftest_exchange(silu_ilu F);
 
 /*
  * Storage layout of the sweep factors (no counterpart in the paper, whose

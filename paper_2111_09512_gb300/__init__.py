@@ -125,6 +125,7 @@ def load():
         "silu_ctx_launch_count": (i32, [vp, ctypes.POINTER(i64)]),
         "silu_ctx_check": (i32, [vp]),
         "silu_ctx_selftest_timeout": (i32, [vp, i32]),
+        "silu_ilu_selftest_exchange": (i32, [vp]),
         "silu_ilu_set_kernel": (i32, [vp, i32]),
         "silu_ilu_set_direct": (i32, [vp, i32]),
         "silu_ilu_set_fused": (i32, [vp, i32]),
@@ -165,7 +166,7 @@ def exported_symbols():
             "silu_amg_level_ilu", "silu_amg_stats", "silu_amg_export_level", "silu_schur_setup", "silu_schur_smooth",
             "silu_schur_stats", "silu_schur_set_interface_prec",
             "silu_ilu_destroy", "silu_ilu_set_lanes", "silu_ctx_profile", "silu_ctx_profile_read",
-            "silu_ctx_launch_count", "silu_ctx_check", "silu_ctx_selftest_timeout", "silu_ilu_set_kernel", "silu_ilu_set_direct", "silu_ilu_set_fused", "silu_ilu_layout", "silu_ilu_tune_table", "silu_ctx_set_overlap",
+            "silu_ctx_launch_count", "silu_ctx_check", "silu_ctx_selftest_timeout", "silu_ilu_selftest_exchange", "silu_ilu_set_kernel", "silu_ilu_set_direct", "silu_ilu_set_fused", "silu_ilu_layout", "silu_ilu_tune_table", "silu_ctx_set_overlap",
             "silu_ctx_set_l2_reuse",
             "silu_smooth_noalloc",
             "silu_batch_setup", "silu_batch_info", "silu_batch_smooth", "silu_batch_fgmres", "silu_batch_destroy",
@@ -510,6 +511,11 @@ class ILU:
 
     def reserve(self, nrhs: int = 1, restart: int = 0):
         _check(self.ctx.handle, load().silu_ilu_reserve(self.handle, nrhs, restart), "silu_ilu_reserve")
+
+    def selftest_exchange(self):
+        """Let a wait of the Arnoldi step's exchange run out (the next check() reports ERR_TIMEOUT) and leave
+        stale entries in its buffer."""
+        _check(self.ctx.handle, load().silu_ilu_selftest_exchange(self.handle), "silu_ilu_selftest_exchange")
 
     def set_kernel(self, variant: int):
         """0 automatic, 1 lanes-per-row kernel, 2 staged (bulk-copy) kernel where it applies (natural

@@ -241,7 +241,6 @@ cudaError_t allocate_krylov(silu_ilu F, int m) {
   if ((e = w.part1.ensure(sizeof(double) * 1024)) != cudaSuccess) return e;
   if ((e = w.scal.ensure(sizeof(double) * 8)) != cudaSuccess) return e;
   if ((e = w.arn.ensure(silu::arnoldi_bytes((int)n))) != cudaSuccess) return e;
-  if ((e = cudaMemsetAsync(w.arn.p, 0, w.arn.bytes, F->ctx->stream)) != cudaSuccess) return e;
   w.restart = m;
   return cudaSuccess;
 }
@@ -1291,6 +1290,22 @@ silu_status silu_ctx_selftest_timeout(silu_ctx ctx, int timeout_ms) {
   return SILU_OK;
 }
 
+silu_status silu_ilu_selftest_exchange(silu_ilu F) {
+  if (!F) return SILU_ERR_INVALID_ARG;
+  silu_ctx ctx = F->ctx;
+  silu_status ds = device_ok(ctx);
+  if (ds != SILU_OK) return ds;
+  if (F->F.L.n == 0) return SILU_OK;
+  try {
+    CK(ensure_krylov(F, std::max(1, F->ws.restart)));
+    LAUNCH(ctx, SILU_K_KRYLOV,
+           silu::launch_exchange_selftest((int)F->F.L.n, F->ws.arn.p, ctx->env.err, ctx->stream));
+  } catch (const CudaFail& f) {
+    return cuda_err(ctx, f.e, f.what);
+  }
+  return SILU_OK;
+}
+
 silu_status silu_ilu_set_kernel(silu_ilu F, int variant) {
   if (!F) return SILU_ERR_INVALID_ARG;
   if (variant < 0 || variant > 3) return set_err(F->ctx, SILU_ERR_INVALID_ARG, "variant must be 0, 1, 2 or 3");
@@ -1825,6 +1840,7 @@ silu_status fgmres_solve(silu_ilu F, double* x, const double* b, double tol, int
       }
       CK(cudaMemsetAsync(g, 0, sizeof(double) * (size_t)(m + 1), s));
       CK(cudaMemsetAsync(H, 0, sizeof(double) * (size_t)(m + 1) * (size_t)m, s));
+      CK(silu::arnoldi_reset(n, m, W.arn.p, ctx->env, s));
       LAUNCH(F->ctx, SILU_K_KRYLOV, silu::launch_normalize(n, part[0], g, V, V, s));
       // Inner iterations run one ahead of the host: iteration j + 1 is queued
       // before the host reads |g_{j+1}| and h_{j+1,j} of iteration j (copied

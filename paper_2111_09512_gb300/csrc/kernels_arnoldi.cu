@@ -17,9 +17,11 @@
 // The exchange: every block publishes its partial sums and every block reads
 // all of them.  An entry is two 8-byte words, each holding half of the FP64
 // value and a 32-bit tag that numbers the exchange, so an entry is complete
-// when both tags match and no fence or atomic is needed.  Tags never repeat
-// between launches: they start at a counter in device memory that block 0
-// advances once its first exchange shows that every block has read it.  Two
+// when both tags match and no fence or atomic is needed.  The j + 2 exchanges of
+// step j have numbers of their own within a restart cycle, known to the host
+// (exchange_number), and the entries are zeroed at the start of each cycle
+// (arnoldi_reset), so nothing that an earlier cycle or solve left behind, one
+// that gave up included, carries a number that is waited for.  Two
 // buffers alternate; a block writes a buffer again only after an exchange
 // through the other one, which every block enters after leaving the first.
 // Every wait is bounded (2 s); one that gives up sets bit 4 (value 16) of the
@@ -58,9 +60,13 @@ struct ArnoldiArgs {
   double* res;
   ulonglong2* entries;  // two buffers of `cap` entries
   int cap;
-  unsigned* counter;
+  unsigned tag;  // number of this step's first exchange
   int* err;
 };
+
+// Number of the first exchange of step j: steps 0 .. j - 1 have i + 2 each, and
+// 0 is an entry that nothing has been written to.
+__host__ __device__ constexpr unsigned exchange_number(int j) { return 1u + (unsigned)j * ((unsigned)j + 3u) / 2u; }
 
 // r[q] holds lane values of warp q (q < 8): the sum over each warp's lanes by
 // the tree of arn_warp_sum, the trees sharing the lanes of one warp (a lane
@@ -182,12 +188,8 @@ __global__ void __launch_bounds__(GB * 256, 1) k_arnoldi(ArnoldiArgs a) {
   const bool lead = blockIdx.x == 0;
   ArnoldiRows rows(a, group, threadIdx.x & 255);
   bool alive = true;
-  unsigned tag = 0;
-  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(tag) : "l"(a.counter) : "memory");
-  const unsigned first = tag;
-  ++tag;  // the buffers start zeroed: no exchange has number 0 before the counter wraps
+  unsigned tag = a.tag;
   if (lead) load_rotations(a, sh, T);
-  __syncthreads();
   // publish the groups' parts of the sum over all rows of the threads' acc
   auto give = [&](double acc, int step) {
     lanes[threadIdx.x] = acc;
@@ -233,11 +235,7 @@ __global__ void __launch_bounds__(GB * 256, 1) k_arnoldi(ArnoldiArgs a) {
     const bool more = i < a.j;
     if (more) rows.load(a.V + (size_t)(i + 1) * (size_t)a.n, rows.nx);
     const double h = take(i);
-    if (lead && threadIdx.x == 0) {
-      sh[i] = h;
-      // every block has read the counter: it has published
-      if (i == 0) *a.counter = first + (unsigned)a.j + 2u;
-    }
+    if (lead && threadIdx.x == 0) sh[i] = h;
     give(rows.step(h, more), i + 1);
   }
   const double h = sqrt(take(a.j + 1));
@@ -306,6 +304,18 @@ __global__ void __launch_bounds__(256, 1) k_arnoldi_cluster(ArnoldiArgs a) {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// What a step that gave up may leave behind: a wait that runs out (no exchange
+// has this number), then entries numbered as the next cycle's first step
+// numbers its own, with values that no sum survives.
+__global__ void k_exchange_selftest(ulonglong2* entries, int cap, int* err) {
+  bool alive = true;
+  double v[1];
+  if (threadIdx.x == 0) collect<1>(entries, 1, 1, ~0u, v, alive, err);
+  __syncthreads();
+  for (int i = threadIdx.x; i < 2 * cap; i += blockDim.x)
+    publish(entries + i, __longlong_as_double(0x7ff8000000000000ll), exchange_number(0) + (i < cap ? 0u : 1u));
+}
+
 template <int GB>
 cudaError_t launch_groups(const ArnoldiArgs& a, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
@@ -367,9 +377,16 @@ int arnoldi_form(int np, const LaunchEnv& env) {
 
 }  // namespace
 
-size_t arnoldi_bytes(int n) {
-  const int np = krylov_parts(n);
-  return 2 * sizeof(ulonglong2) * (size_t)np + 16;
+size_t arnoldi_bytes(int n) { return 2 * sizeof(ulonglong2) * (size_t)krylov_parts(n); }
+
+cudaError_t arnoldi_reset(int n, int m, void* scratch, const LaunchEnv& env, cudaStream_t s) {
+  if (!arnoldi_fits(n, m, env) || arnoldi_form(krylov_parts(n), env) > 0) return cudaSuccess;
+  return cudaMemsetAsync(scratch, 0, arnoldi_bytes(n), s);
+}
+
+cudaError_t launch_exchange_selftest(int n, void* scratch, int* err, cudaStream_t s) {
+  k_exchange_selftest<<<1, 256, 0, s>>>((ulonglong2*)scratch, krylov_parts(n), err);
+  return cudaGetLastError();
 }
 
 cudaError_t arnoldi_prepare(LaunchEnv& env) {
@@ -410,7 +427,7 @@ cudaError_t launch_arnoldi(int n, int j, int m, const double* w, double* V, doub
   a.res = res;
   a.cap = a.np;
   a.entries = (ulonglong2*)scratch;
-  a.counter = (unsigned*)(a.entries + 2 * (size_t)a.cap);
+  a.tag = exchange_number(j);
   a.err = env.err;
   switch (arnoldi_form(a.np, env)) {
     case -1: return launch_groups<1>(a, s);

@@ -35,10 +35,15 @@ cudaError_t launch_mr_step(int n, const double* part_num, const double* part_den
 // of V (stride n) by modified Gram-Schmidt, column j of H, V_{j+1} and the
 // Givens update, with the bits of launch_dot_part, launch_mgs_step,
 // launch_normalize_givens; w is only read.  scratch:
-// arnoldi_bytes(n), zeroed once, this launch's alone.  For sizes and restart
-// lengths that fit (arnoldi_fits); a wait that gives up sets value 16 of
-// *env.err.
+// arnoldi_bytes(n), this workspace's alone.  For sizes and restart lengths
+// that fit (arnoldi_fits); a wait that gives up sets value 16 of *env.err.
+// Each j runs at most once between two calls of arnoldi_reset, which belongs
+// at the start of every restart cycle.
 size_t arnoldi_bytes(int n);
+cudaError_t arnoldi_reset(int n, int m, void* scratch, const LaunchEnv& env, cudaStream_t s);
+// Make a wait of the exchange run out and leave entries in scratch that the
+// next cycle's first step would take for its own.
+cudaError_t launch_exchange_selftest(int n, void* scratch, int* err, cudaStream_t s);
 cudaError_t arnoldi_prepare(LaunchEnv& env);
 bool arnoldi_fits(int n, int m, const LaunchEnv& env);
 cudaError_t launch_arnoldi(int n, int j, int m, const double* w, double* V, double* H, double* cs, double* sn,

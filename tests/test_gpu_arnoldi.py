@@ -133,3 +133,27 @@ def test_arnoldi_grids_of_several_streams_run_side_by_side(silu):
     torch.cuda.synchronize()
     for job, want in zip(jobs, alone):
         assert torch.equal(job[3], want)
+
+
+@pytest.mark.parametrize("size", [(32, 32, 32), (68, 68, 67), (98, 98, 97)], ids=["cluster", "one group", "three groups"])
+def test_solve_after_a_step_that_gave_up(silu, size):
+    """A wait of the exchange that runs out is reported; entries it leaves, numbered like the next solve's, are not
+    read by that solve, which gives the bits of one before."""
+    ctx = silu.Context(0, torch.cuda.current_stream())
+    A = synth.poisson7(*size)
+    n = len(A[0]) - 1
+    F = silu.ilu_setup(ctx, silu.Matrix(ctx, *A), "ilu0")
+    b = torch.from_numpy(synth.rhs(n, 1, seed=3)[:, 0]).cuda()
+    out = []
+    for gave_up in (False, True, True):
+        if gave_up:
+            F.selftest_exchange()
+            with pytest.raises(silu.SiluError) as e:
+                ctx.check()
+            assert e.value.status == silu.ERR_TIMEOUT
+        x = torch.zeros_like(b)
+        st, its, _ = silu.fgmres_solve(F, x, b, tol=0.0, restart=5, maxit=12, sweeps_L=3, sweeps_U=3)
+        ctx.check()
+        assert st == silu.ERR_NOT_CONVERGED and its == 12
+        out.append(x)
+    assert torch.equal(out[0], out[1]) and torch.equal(out[0], out[2])
