@@ -191,6 +191,13 @@ silu_status silu_ctx_check(silu_ctx ctx);
  * stays usable.  Nothing faults, traps or hangs.  Asynchronous.
  */
 silu_status silu_ctx_selftest_timeout(silu_ctx ctx, int timeout_ms);
+/*
+ * Self-test of the out-of-memory paths: from now on, device allocations of
+ * the library's matrices, factors and workspaces made by the calling thread
+ * fail where they would take all such memory of the process beyond `limit`
+ * bytes (negative: no limit).  *in_use (may be NULL): that memory now.
+ */
+silu_status silu_selftest_memory(int64_t limit, int64_t* in_use);
 /* Message of the last failed call on ctx ("" if none); valid until the next call. */
 const char* silu_last_error(silu_ctx ctx);
 /* Library version string. */

@@ -126,6 +126,7 @@ def load():
         "silu_ctx_check": (i32, [vp]),
         "silu_ctx_selftest_timeout": (i32, [vp, i32]),
         "silu_ilu_selftest_exchange": (i32, [vp]),
+        "silu_selftest_memory": (i32, [i64, ctypes.POINTER(i64)]),
         "silu_ilu_set_kernel": (i32, [vp, i32]),
         "silu_ilu_set_direct": (i32, [vp, i32]),
         "silu_ilu_set_fused": (i32, [vp, i32]),
@@ -166,7 +167,7 @@ def exported_symbols():
             "silu_amg_level_ilu", "silu_amg_stats", "silu_amg_export_level", "silu_schur_setup", "silu_schur_smooth",
             "silu_schur_stats", "silu_schur_set_interface_prec",
             "silu_ilu_destroy", "silu_ilu_set_lanes", "silu_ctx_profile", "silu_ctx_profile_read",
-            "silu_ctx_launch_count", "silu_ctx_check", "silu_ctx_selftest_timeout", "silu_ilu_selftest_exchange", "silu_ilu_set_kernel", "silu_ilu_set_direct", "silu_ilu_set_fused", "silu_ilu_layout", "silu_ilu_tune_table", "silu_ctx_set_overlap",
+            "silu_ctx_launch_count", "silu_ctx_check", "silu_ctx_selftest_timeout", "silu_ilu_selftest_exchange", "silu_selftest_memory", "silu_ilu_set_kernel", "silu_ilu_set_direct", "silu_ilu_set_fused", "silu_ilu_layout", "silu_ilu_tune_table", "silu_ctx_set_overlap",
             "silu_ctx_set_l2_reuse",
             "silu_smooth_noalloc",
             "silu_batch_setup", "silu_batch_info", "silu_batch_smooth", "silu_batch_fgmres", "silu_batch_destroy",
@@ -708,6 +709,14 @@ def silu_version() -> str:
 
 def silu_ctx_create(device: int = 0, stream=None) -> Context:
     return Context(device, stream)
+
+
+def silu_selftest_memory(limit: int = -1) -> int:
+    """Let the library's device allocations by this thread fail beyond `limit` bytes in use (negative: no limit);
+    the bytes in use now."""
+    used = ctypes.c_int64()
+    load().silu_selftest_memory(int(limit), ctypes.byref(used))
+    return used.value
 
 
 def silu_mat_create(ctx: Context, row_ptr, col_idx, val) -> Matrix:

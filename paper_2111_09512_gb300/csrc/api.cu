@@ -1,5 +1,6 @@
 // C ABI of libsilu (declared in include/silu.h): handles, host setup and
 // the stream-ordered orchestration of the device kernels.
+#include <atomic>
 #include <cstdio>
 
 #include "internal.h"
@@ -11,6 +12,26 @@ namespace silu {
 int auto_tile_nnz(const Csr& T, bool fp32, int lanes, int passes) {
   return (!fp32 && lanes == 1 && passes == 1 && silu::narrow_fits(T.rp.data(), T.n)) ? silu::kTileNnzNarrow
                                                                                       : silu::kTileNnz;
+}
+
+namespace {
+
+std::atomic<int64_t> g_device_bytes{0};
+thread_local int64_t t_device_limit = INT64_MAX;
+
+}  // namespace
+
+cudaError_t device_alloc(void** p, size_t bytes) {
+  *p = nullptr;
+  if (g_device_bytes.load() + (int64_t)bytes > t_device_limit) return cudaErrorMemoryAllocation;
+  const cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaSuccess) g_device_bytes += (int64_t)bytes;
+  return e;
+}
+
+void device_free(void* p, size_t bytes) {
+  cudaFree(p);
+  g_device_bytes -= (int64_t)bytes;
 }
 
 // Uploads T (row pointers, columns, values in FP64 or FP32) as
@@ -140,6 +161,24 @@ cudaError_t upload_sorted(const Csr& T, bool fp32, SortedBufs& b, DevCsr& d, cud
 
 namespace {
 
+// The tiles tl in a new buffer that takes the old one's place (queued work may
+// still read the old one, and T keeps it if there is no room).
+cudaError_t replace_tiles(DBuf& tiles, const std::vector<int>& tl, DevCsr& T, int lanes, int passes, int max_nnz,
+                          cudaStream_t s) {
+  DBuf nt;
+  cudaError_t e = upload(nt, tl.data(), tl.size(), s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e != cudaSuccess) return e;
+  std::swap(tiles.p, nt.p);
+  std::swap(tiles.bytes, nt.bytes);
+  T.tiles = tiles.as<int4>();
+  T.ntiles = (int)(tl.size() / 4);
+  T.tile_lanes = lanes;
+  T.tile_passes = passes;
+  T.tile_nnz = max_nnz;
+  return cudaSuccess;
+}
+
 // Re-apply a launch shape kept from before an upload: tiles for g lanes per
 // row and rl rows per lane, gather width.
 cudaError_t keep_shape(const Csr& h, DBuf& tiles, DevCsr& T, const DevCsr& old, cudaStream_t s) {
@@ -152,16 +191,7 @@ cudaError_t keep_shape(const Csr& h, DBuf& tiles, DevCsr& T, const DevCsr& old, 
                                                                                                  : old.tile_nnz;
   std::vector<int> tl;
   if (!silu::make_tiles(h.rp.data(), h.n, old.tile_lanes, old.tile_passes, tl, lim)) return cudaSuccess;
-  cudaError_t e = upload(tiles, tl.data(), tl.size(), s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e == cudaSuccess) {
-    T.tiles = tiles.as<int4>();
-    T.ntiles = (int)(tl.size() / 4);
-    T.tile_lanes = old.tile_lanes;
-    T.tile_passes = old.tile_passes;
-    T.tile_nnz = lim;
-  }
-  return e;
+  return replace_tiles(tiles, tl, T, old.tile_lanes, old.tile_passes, lim, s);
 }
 
 }  // namespace
@@ -214,6 +244,7 @@ cudaError_t allocate_vectors(silu_ilu F, int nrhs) {
   Workspace& w = F->ws;
   if (bytes <= w.vec_bytes && w.r.p) return cudaSuccess;
   w.drop_graphs();
+  w.vec_bytes = 0;  // until all four are there
   cudaError_t e;
   if ((e = w.r.ensure(bytes)) != cudaSuccess) return e;
   if ((e = w.c.ensure(bytes)) != cudaSuccess) return e;
@@ -227,6 +258,7 @@ cudaError_t allocate_krylov(silu_ilu F, int m) {
   Workspace& w = F->ws;
   if (m <= w.restart && w.V.p) return cudaSuccess;
   w.drop_graphs();
+  w.restart = 0;  // until all of them are there
   const size_t n = (size_t)F->F.L.n;
   cudaError_t e;
   if ((e = w.V.ensure(sizeof(double) * n * (size_t)(m + 1))) != cudaSuccess) return e;
@@ -1141,16 +1173,7 @@ namespace {
 cudaError_t retile(const Csr& h, DBuf& tiles, DevCsr& T, int g, int rl, cudaStream_t s, int max_nnz) {
   std::vector<int> tl;
   if (!silu::make_tiles(h.rp.data(), h.n, g, rl, tl, max_nnz)) return cudaSuccess;  // keeps the current tiles
-  cudaError_t e = upload(tiles, tl.data(), tl.size(), s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e == cudaSuccess) {
-    T.tiles = tiles.as<int4>();
-    T.ntiles = (int)(tl.size() / 4);
-    T.tile_lanes = g;
-    T.tile_passes = rl;
-    T.tile_nnz = max_nnz;
-  }
-  return e;
+  return replace_tiles(tiles, tl, T, g, rl, max_nnz, s);
 }
 
 // Tile limit of an autotuner candidate's gather width: 0 automatic (narrow
@@ -1290,6 +1313,12 @@ silu_status silu_ctx_selftest_timeout(silu_ctx ctx, int timeout_ms) {
   return SILU_OK;
 }
 
+silu_status silu_selftest_memory(int64_t limit, int64_t* in_use) {
+  silu::t_device_limit = limit < 0 ? INT64_MAX : limit;
+  if (in_use) *in_use = silu::g_device_bytes.load();
+  return SILU_OK;
+}
+
 silu_status silu_ilu_selftest_exchange(silu_ilu F) {
   if (!F) return SILU_ERR_INVALID_ARG;
   silu_ctx ctx = F->ctx;
@@ -1415,18 +1444,8 @@ silu_status silu_mat_set_shape(silu_mat A, int lanes, int passes, int chunk) {
   std::vector<int> tl;
   if (!silu::make_tiles(A->A.rp.data(), A->A.n, g, rl, tl, lim))
     return set_err(ctx, SILU_ERR_INVALID_ARG, "a row is too long for the staged kernel");
-  // new tiles in a new buffer (the old one may still be read by queued work)
-  DBuf nt;
-  cudaError_t e = upload(nt, tl.data(), tl.size(), ctx->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+  const cudaError_t e = replace_tiles(A->tiles, tl, A->d, g, rl, lim, ctx->stream);
   if (e != cudaSuccess) return cuda_err(ctx, e, "upload of the tiles");
-  std::swap(A->tiles.p, nt.p);
-  std::swap(A->tiles.bytes, nt.bytes);
-  A->d.tiles = A->tiles.as<int4>();
-  A->d.ntiles = (int)(tl.size() / 4);
-  A->d.tile_lanes = g;
-  A->d.tile_passes = rl;
-  A->d.tile_nnz = lim;
   A->d.chunk = (chunk == 8) ? 8 : 16;
   A->d.explicit_shape = lanes != 0 || passes != 0 || chunk != 0;  // (0, 0, 0): the sliced copy where there is one
   A->gen++;

@@ -356,6 +356,7 @@ cudaError_t allocate_bkrylov(silu_batch B, int m) {
   for (InnerGraph& ig : B->graphs)
     if (ig.exec) cudaGraphExecDestroy(ig.exec);
   B->graphs.clear();
+  B->restart = 0;  // until all buffers are there
   const size_t N = (size_t)B->offsets.back();
   const size_t ns = (size_t)B->count;
   cudaError_t e;

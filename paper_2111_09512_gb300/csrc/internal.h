@@ -23,6 +23,11 @@
 
 namespace silu {
 
+// Device memory of the library's objects, counted over the process, and
+// refused beyond the calling thread's limit (silu_selftest_memory).
+cudaError_t device_alloc(void** p, size_t bytes);
+void device_free(void* p, size_t bytes);
+
 // Owning device buffer.
 struct DBuf {
   void* p = nullptr;
@@ -32,15 +37,17 @@ struct DBuf {
   DBuf& operator=(const DBuf&) = delete;
   ~DBuf() { release(); }
   void release() {
-    if (p) cudaFree(p);
+    if (p) device_free(p, bytes);
     p = nullptr;
     bytes = 0;
   }
+  // At least b bytes; the contents are lost when the buffer has to grow, and
+  // the buffer is empty when that fails.
   cudaError_t ensure(size_t b) {
     if (b <= bytes && p) return cudaSuccess;
     release();
     if (b == 0) b = 16;
-    cudaError_t e = cudaMalloc(&p, b);
+    cudaError_t e = device_alloc(&p, b);
     if (e != cudaSuccess) {
       p = nullptr;
       return e;
