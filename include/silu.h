@@ -160,6 +160,20 @@ silu_status silu_ctx_profile_read(silu_ctx ctx, int kclass, int64_t* launches, d
  */
 silu_status silu_ctx_set_overlap(silu_ctx ctx, int enable);
 /*
+ * Sliced copies.  Sweeps and products run on a second copy of each matrix,
+ * factor and hierarchy operator, padded to slices of 32 rows (see
+ * silu_ilu_set_kernel), beside its CSR arrays: 10 bytes per padded entry in
+ * FP64 and 6 in FP32 (14 and 8 where columns do not fit 16-bit offsets), at
+ * most 1.4 padded entries per entry.  They give way when memory runs out: a
+ * call on the context whose own allocations fail gives up all copies of the
+ * context's objects and tries again without building any.  For memory that
+ * the caller wants for itself: enable = 0 gives up the copies now and builds
+ * none from here on (the sweeps run on the CSR tiles, for one right-hand side
+ * with the same bits); enable = 1 (default) builds them for objects created
+ * or refactored later.  Blocks.
+ */
+silu_status silu_ctx_set_copies(silu_ctx ctx, int enable);
+/*
  * L2 reuse of staged sweeps (bit flags, default 1; applies to launches and
  * graph captures made after the call).  Bit 0: consecutive staged launches on the
  * context alternate their direction (every other launch walks the row tiles

@@ -126,6 +126,7 @@ def load():
         "silu_ctx_check": (i32, [vp]),
         "silu_ctx_selftest_timeout": (i32, [vp, i32]),
         "silu_ilu_selftest_exchange": (i32, [vp]),
+        "silu_ctx_set_copies": (i32, [vp, i32]),
         "silu_selftest_memory": (i32, [i64, ctypes.POINTER(i64)]),
         "silu_ilu_set_kernel": (i32, [vp, i32]),
         "silu_ilu_set_direct": (i32, [vp, i32]),
@@ -167,7 +168,7 @@ def exported_symbols():
             "silu_amg_level_ilu", "silu_amg_stats", "silu_amg_export_level", "silu_schur_setup", "silu_schur_smooth",
             "silu_schur_stats", "silu_schur_set_interface_prec",
             "silu_ilu_destroy", "silu_ilu_set_lanes", "silu_ctx_profile", "silu_ctx_profile_read",
-            "silu_ctx_launch_count", "silu_ctx_check", "silu_ctx_selftest_timeout", "silu_ilu_selftest_exchange", "silu_selftest_memory", "silu_ilu_set_kernel", "silu_ilu_set_direct", "silu_ilu_set_fused", "silu_ilu_layout", "silu_ilu_tune_table", "silu_ctx_set_overlap",
+            "silu_ctx_launch_count", "silu_ctx_check", "silu_ctx_selftest_timeout", "silu_ilu_selftest_exchange", "silu_selftest_memory", "silu_ctx_set_copies", "silu_ilu_set_kernel", "silu_ilu_set_direct", "silu_ilu_set_fused", "silu_ilu_layout", "silu_ilu_tune_table", "silu_ctx_set_overlap",
             "silu_ctx_set_l2_reuse",
             "silu_smooth_noalloc",
             "silu_batch_setup", "silu_batch_info", "silu_batch_smooth", "silu_batch_fgmres", "silu_batch_destroy",
@@ -223,6 +224,10 @@ class Context:
     def set_overlap(self, enable: bool):
         """Launch each staged sweep as a programmatic dependent of the kernel before it (default on)."""
         _check(self.handle, load().silu_ctx_set_overlap(self.handle, 1 if enable else 0), "silu_ctx_set_overlap")
+
+    def set_copies(self, enable: bool):
+        """Sliced copies of matrices and factors: give them up and build no more (False), or build them (default)."""
+        _check(self.handle, load().silu_ctx_set_copies(self.handle, 1 if enable else 0), "silu_ctx_set_copies")
 
     def set_l2_reuse(self, flags: int):
         """L2 reuse flags of staged sweeps: 1 alternate direction, 2 factor at normal priority, 4 vectors at

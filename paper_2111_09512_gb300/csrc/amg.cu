@@ -139,18 +139,19 @@ double* level_cycle(silu_ilu F, int l, int mL, int mU, bool capturing) {
   return coarse_smooth(F, l, x, b, false, mL, mU, capturing);
 }
 
-cudaError_t upload_level(const silu::AmgLevel& H, AmgDevLevel& D, bool own_a, bool coarsest, bool gs, Copies cp,
-                         cudaStream_t s) {
+cudaError_t upload_level(silu_ctx ctx, const silu::AmgLevel& H, AmgDevLevel& D, bool own_a, bool coarsest, bool gs) {
+  cudaStream_t s = ctx->stream;
+  const Copies cp = ctx->copies;
   cudaError_t e = cudaSuccess;
   D.n = H.A.n;
-  if (own_a) e = silu::upload_csr(H.A, false, D.A_rp, D.A_ci, D.A_va, D.A_tiles, D.A, s, cp);
+  if (own_a) e = silu::upload_csr(ctx, H.A, false, D.A_rp, D.A_ci, D.A_va, D.A_tiles, D.A, cp);
   if (e == cudaSuccess && !coarsest) {
-    e = silu::upload_csr(negated(H.P), false, D.P_rp, D.P_ci, D.P_va, D.P_tiles, D.Pneg, s, cp);
-    if (e == cudaSuccess) e = silu::upload_csr(H.R, false, D.R_rp, D.R_ci, D.R_va, D.R_tiles, D.R, s, cp);
+    e = silu::upload_csr(ctx, negated(H.P), false, D.P_rp, D.P_ci, D.P_va, D.P_tiles, D.Pneg, cp);
+    if (e == cudaSuccess) e = silu::upload_csr(ctx, H.R, false, D.R_rp, D.R_ci, D.R_va, D.R_tiles, D.R, cp);
   }
   if (e == cudaSuccess) e = silu::upload(D.l1inv, H.l1inv.data(), H.l1inv.size(), s);
   if (e == cudaSuccess && gs && own_a) {
-    e = silu::upload_csr(H.Lgs, false, D.G_rp, D.G_ci, D.G_va, D.G_tiles, D.Lgs, s, cp);
+    e = silu::upload_csr(ctx, H.Lgs, false, D.G_rp, D.G_ci, D.G_va, D.G_tiles, D.Lgs, cp);
     if (e == cudaSuccess) e = silu::upload(D.gdinv, H.dinv.data(), H.dinv.size(), s);
   }
   const size_t vb = sizeof(double) * (size_t)std::max<int64_t>(D.n, 1);
@@ -276,13 +277,17 @@ silu_status silu_amg_setup(silu_ilu F, const silu_amg_params* params) {
       cudaStream_t s = ctx->stream;
       const size_t nl = G->host.lev.size();
       cudaError_t e = silu::ensure_vectors(F, 1);
-      for (size_t l = 0; e == cudaSuccess && l < nl; ++l) {
-        G->lev.emplace_back(new AmgDevLevel);
-        e = upload_level(G->host.lev[l], *G->lev[l], l > 0, l + 1 == nl, p.coarse_smoother == SILU_AMG_POLY_GS,
-                         ctx->copies, s);
-      }
       if (e == cudaSuccess)
-        e = silu::upload(G->cinv, G->host.coarse_inv.data(), G->host.coarse_inv.size(), s);
+        e = silu::with_room(ctx, [&] {
+          cudaError_t u = cudaSuccess;
+          G->lev.clear();
+          for (size_t l = 0; u == cudaSuccess && l < nl; ++l) {
+            G->lev.emplace_back(new AmgDevLevel);
+            u = upload_level(ctx, G->host.lev[l], *G->lev[l], l > 0, l + 1 == nl,
+                             p.coarse_smoother == SILU_AMG_POLY_GS);
+          }
+          return u == cudaSuccess ? silu::upload(G->cinv, G->host.coarse_inv.data(), G->host.coarse_inv.size(), s) : u;
+        });
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);
       if (e != cudaSuccess) return silu::cuda_err(ctx, e, "upload of the AMG hierarchy");
       for (silu_ilu FL : G->ilu_fac) {

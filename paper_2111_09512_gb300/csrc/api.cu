@@ -37,8 +37,9 @@ void device_free(void* p, size_t bytes) {
 // Uploads T (row pointers, columns, values in FP64 or FP32) as
 // 16-byte-rounded copies, builds the row tiles of the staged kernel in the
 // automatic launch shape and the sliced copy where it pays (`copies`).
-cudaError_t upload_csr(const silu::Csr& T, bool fp32, DBuf& rp, DBuf& ci, DBuf& va, DBuf& tiles, DevCsr& d,
-                       cudaStream_t s, Copies copies) {
+cudaError_t upload_csr(silu_ctx ctx, const silu::Csr& T, bool fp32, DBuf& rp, DBuf& ci, DBuf& va, DBuf& tiles,
+                       DevCsr& d, Copies copies) {
+  cudaStream_t s = ctx->stream;
   const size_t n = (size_t)T.n, nnz = (size_t)T.nnz();
   const size_t vs = fp32 ? sizeof(float) : sizeof(double);
   std::vector<int32_t> rp32(T.rp.begin(), T.rp.end());
@@ -68,20 +69,29 @@ cudaError_t upload_csr(const silu::Csr& T, bool fp32, DBuf& rp, DBuf& ci, DBuf& 
   d.fp32 = fp32;
   d.explicit_shape = false;
   d.sl.reset();
-  const bool slice = copies != Copies::kCsr && silu::slices_pay(T.rp.data(), T.n, fp32);
-  if (e == cudaSuccess && slice) e = silu::build_slices(T.rp.data(), d, s);
   std::vector<int> tl;
   const int tlanes = silu::staged_lanes(T.rp.data(), T.n);
   const int tpasses = silu::staged_passes(T.rp.data(), T.n, tlanes);
   const int tnnz = auto_tile_nnz(T, fp32, tlanes, tpasses);
   const bool tiled = silu::make_tiles(T.rp.data(), T.n, tlanes, tpasses, tl, tnnz);
   if (e == cudaSuccess && tiled) e = upload(tiles, tl.data(), tl.size(), s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // host staging vectors die at return
   d.tiles = tiled ? tiles.as<int4>() : nullptr;
   d.ntiles = tiled ? (int)(tl.size() / 4) : 0;
   d.tile_lanes = tlanes;
   d.tile_passes = tpasses;
   d.tile_nnz = tnnz;
+  // the sliced copy last, in what memory the arrays above leave
+  const bool slice = copies != Copies::kCsr && !ctx->no_copies && silu::slices_pay(T.rp.data(), T.n, fp32);
+  if (e == cudaSuccess && slice) {
+    e = silu::build_slices(T.rp.data(), d, s);
+    if (e == cudaSuccess && d.sl) {
+      auto& all = ctx->slices;
+      all.erase(std::remove_if(all.begin(), all.end(), [](const auto& w) { return w.expired(); }), all.end());
+      all.push_back(d.sl);
+    }
+  }
+  // host staging vectors die at return, and a sweep reads the matrix ahead of the kernel before it
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e == cudaSuccess && d.sl && copies == Copies::kSmaller) {
     if (tiled && d.sl->bytes > rp.bytes + ci.bytes + va.bytes + tiles.bytes) {
       d.sl.reset();
@@ -91,31 +101,26 @@ cudaError_t upload_csr(const silu::Csr& T, bool fp32, DBuf& rp, DBuf& ci, DBuf& 
       d.va = nullptr;
       d.tiles = nullptr;
       d.ntiles = 0;
+      d.sl->sole = true;
     }
   }
   return e;
 }
 
-// After a failed allocation of F's workspace: drop the sliced copies of F and
-// A, whose sweeps then run on the tiles (the same bits).  False if there was
-// nothing to drop.
-bool drop_slices(silu_ilu F) {
+bool drop_slices(silu_ctx ctx) {
   bool any = false;
-  for (DevCsr* d : {&F->A->d, &F->dL, &F->dU}) {
-    if (!d->sl || !d->rp) continue;
-    d->sl.reset();
+  for (const std::weak_ptr<Slices>& w : ctx->slices) {
+    const std::shared_ptr<Slices> S = w.lock();
+    if (!S || !S->buf || S->sole) continue;
+    S->release();  // waits for the device
     any = true;
   }
-  if (any) {
-    cudaGetLastError();
-    F->ws.drop_graphs();
-    F->config_gen++;
-    F->A->gen++;
-  }
+  if (any) ctx->copies_gen++;
   return any;
 }
 
-cudaError_t upload_sorted(const Csr& T, bool fp32, SortedBufs& b, DevCsr& d, cudaStream_t s) {
+cudaError_t upload_sorted(silu_ctx ctx, const Csr& T, bool fp32, SortedBufs& b, DevCsr& d) {
+  cudaStream_t s = ctx->stream;
   d.srp = nullptr;
   d.sci = nullptr;
   d.sva = nullptr;
@@ -140,7 +145,7 @@ cudaError_t upload_sorted(const Csr& T, bool fp32, SortedBufs& b, DevCsr& d, cud
   S.ci.swap(sci);
   S.va.swap(sva);
   DevCsr sd;
-  cudaError_t e = upload_csr(S, fp32, b.rp, b.ci, b.va, b.tiles, sd, s, Copies::kCsr);
+  cudaError_t e = upload_csr(ctx, S, fp32, b.rp, b.ci, b.va, b.tiles, sd, Copies::kCsr);
   std::vector<int> tl;
   if (e == cudaSuccess && !silu::make_tiles(S.rp.data(), S.n, 1, 1, tl)) return cudaSuccess;
   if (e == cudaSuccess) e = upload(b.tiles, tl.data(), tl.size(), s);
@@ -198,13 +203,14 @@ cudaError_t keep_shape(const Csr& h, DBuf& tiles, DevCsr& T, const DevCsr& old, 
 
 cudaError_t ensure_sorted(silu_ilu F) {
   if (F->sorted_ready) return cudaSuccess;
-  cudaStream_t s = F->ctx->stream;
   const bool f32 = F->prec == SILU_FP32;
   const Csr& Ut = scaled_upper(F) ? F->Us : F->F.U;
   F->ws.drop_graphs();
   F->config_gen++;
-  cudaError_t e = upload_sorted(F->F.L, f32, F->Lsort, F->dL, s);
-  if (e == cudaSuccess) e = upload_sorted(Ut, f32, F->Usort, F->dU, s);
+  const cudaError_t e = with_room(F->ctx, [&] {
+    const cudaError_t el = upload_sorted(F->ctx, F->F.L, f32, F->Lsort, F->dL);
+    return el == cudaSuccess ? upload_sorted(F->ctx, Ut, f32, F->Usort, F->dU) : el;
+  });
   if (e == cudaSuccess) F->sorted_ready = true;
   return e;
 }
@@ -214,12 +220,14 @@ cudaError_t upload_factors(silu_ilu F) {
   const bool f32 = F->prec == SILU_FP32;
   const Csr& Ut = scaled_upper(F) ? F->Us : F->F.U;
   const bool had = F->dL.rp != nullptr;
-  const DevCsr oldL = F->dL, oldU = F->dU;
+  DevCsr oldL = F->dL, oldU = F->dU;  // for their launch shapes
+  oldL.sl.reset();
+  oldU.sl.reset();
   F->ws.drop_graphs();  // captured launches refer to the shapes and arrays replaced here
   F->config_gen++;
   const Copies cp = F->ctx->factor_copies;
-  cudaError_t e = upload_csr(F->F.L, f32, F->L_rp, F->L_ci, F->L_va, F->L_tiles, F->dL, s, cp);
-  if (e == cudaSuccess) e = upload_csr(Ut, f32, F->U_rp, F->U_ci, F->U_va, F->U_tiles, F->dU, s, cp);
+  cudaError_t e = upload_csr(F->ctx, F->F.L, f32, F->L_rp, F->L_ci, F->L_va, F->L_tiles, F->dL, cp);
+  if (e == cudaSuccess) e = upload_csr(F->ctx, Ut, f32, F->U_rp, F->U_ci, F->U_va, F->U_tiles, F->dU, cp);
   if (e == cudaSuccess && F->sorted_ready) {  // sorted copies in use: rebuild them from the new values
     F->sorted_ready = false;
     e = ensure_sorted(F);
@@ -279,15 +287,12 @@ cudaError_t allocate_krylov(silu_ilu F, int m) {
 
 }  // namespace
 
-// The workspace comes before the sliced copies where memory holds only one.
 cudaError_t ensure_vectors(silu_ilu F, int nrhs) {
-  const cudaError_t e = allocate_vectors(F, nrhs);
-  return e == cudaErrorMemoryAllocation && drop_slices(F) ? allocate_vectors(F, nrhs) : e;
+  return with_room(F->ctx, [&] { return allocate_vectors(F, nrhs); });
 }
 
 cudaError_t ensure_krylov(silu_ilu F, int m) {
-  const cudaError_t e = allocate_krylov(F, m);
-  return e == cudaErrorMemoryAllocation && drop_slices(F) ? allocate_krylov(F, m) : e;
+  return with_room(F->ctx, [&] { return allocate_krylov(F, m); });
 }
 
 namespace {
@@ -403,12 +408,14 @@ cudaError_t ensure_tri(silu_ilu F, int R) {
   if (F->tri_state[k].p) return cudaSuccess;
   cudaStream_t s = F->ctx->stream;
   const size_t vb = sizeof(double) * (size_t)std::max<int64_t>(F->F.L.n, 1) * (size_t)R;
-  cudaError_t e = F->tri_y[k].ensure(vb);
-  if (e == cudaSuccess) e = F->tri_v[k].ensure(vb);
+  DBuf st;
+  cudaError_t e = with_room(F->ctx, [&] {
+    cudaError_t a = F->tri_y[k].ensure(vb);
+    if (a == cudaSuccess) a = F->tri_v[k].ensure(vb);
+    return a == cudaSuccess ? st.ensure(4 * sizeof(unsigned)) : a;
+  });
   if (e == cudaSuccess) e = cudaMemsetAsync(F->tri_y[k].p, 0, vb, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(F->tri_v[k].p, 0, vb, s);
-  DBuf st;
-  if (e == cudaSuccess) e = st.ensure(4 * sizeof(unsigned));
   if (e == cudaSuccess) e = cudaMemsetAsync(st.p, 0, 4 * sizeof(unsigned), s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return e;
@@ -459,9 +466,10 @@ cudaError_t decide_direct(silu_ilu F, int R) {
   return e;
 }
 
-cudaError_t ensure_direct(silu_ilu F) {
-  if (F->direct_ready) return cudaSuccess;
-  F->ws.drop_graphs();  // captured solves refer to the arrays uploaded here
+namespace {
+
+// The FP64 factors, level lists and plan of the exact solves.
+cudaError_t upload_direct(silu_ilu F) {
   cudaStream_t s = F->ctx->stream;
   cudaError_t e = cudaSuccess;
   // FP64 L_s: reuse the sweep copy when it is FP64
@@ -476,21 +484,30 @@ cudaError_t ensure_direct(silu_ilu F) {
                           cudaMemcpyHostToDevice, s);
     F->dL64.va = F->L64_va.p;
     F->dL64.fp32 = false;
-    F->dL64.sl.reset();  // an FP32 copy
   }
+  F->dL64.sl.reset();  // the exact solves read the CSR arrays
   if (e != cudaSuccess) return e;
   // FP64 Utilde_s: reuse when the sweeps use it in FP64
   if (F->prec == SILU_FP64 && scaled_upper(F)) {
     F->dS64 = F->dU;
+    F->dS64.sl.reset();
   } else {
-    e = upload_csr(F->Us, false, F->S_rp, F->S_ci, F->S_va, F->S_tiles, F->dS64, s, Copies::kCsr);
+    e = upload_csr(F->ctx, F->Us, false, F->S_rp, F->S_ci, F->S_va, F->S_tiles, F->dS64, Copies::kCsr);
     if (e != cudaSuccess) return e;
   }
   e = upload(F->levLrows_d, F->levLrows.data(), F->levLrows.size(), s);
   if (e == cudaSuccess) e = upload(F->levUrows_d, F->levUrows.data(), F->levUrows.size(), s);
   if (e == cudaSuccess) e = build_tri_plan(F);
+  return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
+}
+
+}  // namespace
+
+cudaError_t ensure_direct(silu_ilu F) {
+  if (F->direct_ready) return cudaSuccess;
+  F->ws.drop_graphs();  // captured solves refer to the arrays uploaded here
+  cudaError_t e = with_room(F->ctx, [&] { return upload_direct(F); });
   if (e == cudaSuccess) e = ensure_tri(F, 1);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e == cudaSuccess) F->direct_ready = true;
   for (int& c : F->direct_choice) c = 0;  // the factors changed: decide again
   if (e == cudaSuccess) e = decide_direct(F, 1);
@@ -518,7 +535,7 @@ bool small_block(silu_ilu F, int R) {
 // factors, an explicit staged variant (2, 3) keep the tiles; variant 1 keeps
 // the lanes-per-row kernel everywhere.
 bool use_slices(silu_ilu F, const DevCsr& T, int R, int ldx) {
-  if (!T.sl || T.explicit_shape || F->variant == 1 || R > 4 || (R == 1 && ldx != 1)) return false;
+  if (!T.sliced() || T.explicit_shape || F->variant == 1 || R > 4 || (R == 1 && ldx != 1)) return false;
   if (F->variant != 0 && (&T == &F->dL || &T == &F->dU)) return false;
   // Large matrices that the tiled sweeps serve faster (per sweep, slices
   // against tiles):
@@ -965,7 +982,7 @@ void fgmres_inner_graph(silu_ilu F, int j, int m, int mL, int mU, int precond) {
   silu_ctx ctx = F->ctx;
   for (KrylovGraph& kg : F->ws.kgraphs)
     if (kg.j == j && kg.m == m && kg.mL == mL && kg.mU == mU && kg.precond == precond && kg.gen == F->config_gen &&
-        kg.agen == F->A->gen) {
+        kg.agen == F->A->gen && kg.cgen == ctx->copies_gen) {
       ctx->launches += kg.kernels;
       CK(cudaGraphLaunch(kg.exec, ctx->stream));
       return;
@@ -998,6 +1015,7 @@ void fgmres_inner_graph(silu_ilu F, int j, int m, int mL, int mU, int precond) {
   kg.precond = precond;
   kg.gen = F->config_gen;
   kg.agen = F->A->gen;
+  kg.cgen = ctx->copies_gen;
   kg.kernels = ctx->launches - l0;
   ctx->launches = l0;
   if (e == cudaSuccess) e = cudaGraphInstantiate(&kg.exec, graph, 0);
@@ -1018,6 +1036,15 @@ int scale_upper(silu_ilu F, std::string& msg) {
     return silu::rowcol_scale(F->F.U, kRuizMaxit, kRuizTol, F->Us, F->dinv, F->dcol, F->ruiz_steps, msg);
   F->dcol.clear();
   return silu::row_scale(F->F.U, F->Us, F->dinv, msg);
+}
+
+// The factors and their scaling (on the context's stream).
+cudaError_t upload_solver(silu_ilu F) {
+  cudaStream_t s = F->ctx->stream;
+  cudaError_t e = upload_factors(F);
+  if (e == cudaSuccess) e = upload(F->d_dinv, F->dinv.data(), F->dinv.size(), s);
+  if (e == cudaSuccess && !F->dcol.empty()) e = upload(F->d_dcol, F->dcol.data(), F->dcol.size(), s);
+  return e;
 }
 
 silu_status finish_setup(silu_ilu F) {
@@ -1047,9 +1074,7 @@ silu_status finish_setup(silu_ilu F) {
     silu_status ds = device_ok(ctx);
     if (ds != SILU_OK) return ds;
     cudaStream_t s = ctx->stream;
-    cudaError_t e = upload_factors(F);
-    if (e == cudaSuccess) e = upload(F->d_dinv, F->dinv.data(), F->dinv.size(), s);
-    if (e == cudaSuccess && !F->dcol.empty()) e = upload(F->d_dcol, F->dcol.data(), F->dcol.size(), s);
+    cudaError_t e = with_room(ctx, [&] { return upload_solver(F); });
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_err(ctx, e, "upload of the factors");
   }
@@ -1117,6 +1142,14 @@ silu_status silu_ctx_profile(silu_ctx ctx, int enable) {
 silu_status silu_ctx_set_overlap(silu_ctx ctx, int enable) {
   if (!ctx) return SILU_ERR_INVALID_ARG;
   ctx->env.overlap = enable != 0;
+  return SILU_OK;
+}
+
+silu_status silu_ctx_set_copies(silu_ctx ctx, int enable) {
+  silu_status ds = device_ok(ctx);
+  if (ds != SILU_OK) return ds;
+  ctx->no_copies = enable == 0;
+  if (!enable) drop_slices(ctx);
   return SILU_OK;
 }
 
@@ -1221,8 +1254,10 @@ silu_status silu_ilu_autotune(silu_ilu F, int sweeps_L, int sweeps_U, int* choic
   int best = 0;
   double best_ms = 1e300;
   try {
-    CK(x.ensure(sizeof(double) * n));
-    CK(b.ensure(sizeof(double) * n));
+    CK(with_room(ctx, [&] {
+      const cudaError_t e = x.ensure(sizeof(double) * n);
+      return e == cudaSuccess ? b.ensure(sizeof(double) * n) : e;
+    }));
     CK(cudaMemsetAsync(b.p, 0, sizeof(double) * n, s));
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
@@ -1243,8 +1278,12 @@ silu_status silu_ilu_autotune(silu_ilu F, int sweeps_L, int sweeps_U, int* choic
         const int pU = c.passes ? c.passes : silu::staged_passes(Ut.rp.data(), Ut.n, gU);
         const bool f32 = F->prec == SILU_FP32;
         const int rlL = gL == 1 ? pL : 1, rlU = gU == 1 ? pU : 1;
-        CK(retile(F->F.L, F->L_tiles, F->dL, gL, rlL, s, candidate_tile_nnz(F->F.L, f32, gL, rlL, c.chunk)));
-        CK(retile(Ut, F->U_tiles, F->dU, gU, rlU, s, candidate_tile_nnz(Ut, f32, gU, rlU, c.chunk)));
+        CK(with_room(ctx, [&] {
+          return retile(F->F.L, F->L_tiles, F->dL, gL, rlL, s, candidate_tile_nnz(F->F.L, f32, gL, rlL, c.chunk));
+        }));
+        CK(with_room(ctx, [&] {
+          return retile(Ut, F->U_tiles, F->dU, gU, rlU, s, candidate_tile_nnz(Ut, f32, gU, rlU, c.chunk));
+        }));
         F->dL.chunk = F->dU.chunk = (c.chunk == 8) ? 8 : 16;
       }
     };
@@ -1409,7 +1448,8 @@ silu_status silu_mat_create(silu_ctx ctx, int64_t n, int64_t nnz, const int64_t*
         delete M;
         return ds;
       }
-      cudaError_t e = upload_csr(M->A, false, M->rp, M->ci, M->va, M->tiles, M->d, ctx->stream, ctx->copies);
+      cudaError_t e = with_room(
+          ctx, [&] { return upload_csr(ctx, M->A, false, M->rp, M->ci, M->va, M->tiles, M->d, ctx->copies); });
       if (e != cudaSuccess) {
         delete M;
         return cuda_err(ctx, e, "upload of A");
@@ -1444,7 +1484,8 @@ silu_status silu_mat_set_shape(silu_mat A, int lanes, int passes, int chunk) {
   std::vector<int> tl;
   if (!silu::make_tiles(A->A.rp.data(), A->A.n, g, rl, tl, lim))
     return set_err(ctx, SILU_ERR_INVALID_ARG, "a row is too long for the staged kernel");
-  const cudaError_t e = replace_tiles(A->tiles, tl, A->d, g, rl, lim, ctx->stream);
+  const cudaError_t e =
+      with_room(ctx, [&] { return replace_tiles(A->tiles, tl, A->d, g, rl, lim, ctx->stream); });
   if (e != cudaSuccess) return cuda_err(ctx, e, "upload of the tiles");
   A->d.chunk = (chunk == 8) ? 8 : 16;
   A->d.explicit_shape = lanes != 0 || passes != 0 || chunk != 0;  // (0, 0, 0): the sliced copy where there is one
@@ -1469,9 +1510,11 @@ silu_status silu_mat_autotune(silu_mat A, int* lanes, int* passes, int* chunk, d
     DBuf x, b, r;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     try {
-      CK(x.ensure(sizeof(double) * n));
-      CK(b.ensure(sizeof(double) * n));
-      CK(r.ensure(sizeof(double) * n));
+      CK(with_room(ctx, [&] {
+        cudaError_t e = x.ensure(sizeof(double) * n);
+        if (e == cudaSuccess) e = b.ensure(sizeof(double) * n);
+        return e == cudaSuccess ? r.ensure(sizeof(double) * n) : e;
+      }));
       CK(cudaMemsetAsync(x.p, 0, sizeof(double) * n, s));
       CK(cudaMemsetAsync(b.p, 0, sizeof(double) * n, s));
       CK(cudaEventCreate(&e0));
@@ -1525,7 +1568,7 @@ silu_status silu_mat_residual(silu_mat A, double* r, const double* x, const doub
   if (A->A.n == 0) return SILU_OK;
   cudaStream_t s = ctx->stream;
   try {
-    if (A->d.sl && !A->d.explicit_shape) {
+    if (A->d.sliced() && !A->d.explicit_shape) {
       for (int c0 = 0; c0 < nrhs;) {
         const int w = slice_width(nrhs - c0);
         LAUNCH(ctx, SILU_K_RESIDUAL, silu::launch_sweep_slices(A->d, silu::MODE_D, ctx->env, w, nrhs, b + c0, x + c0,
@@ -1711,9 +1754,7 @@ silu_status ilu_refactor(silu_ilu F, const double* new_val) {
       cudaStream_t s = ctx->stream;
       cudaError_t e = upload(F->A->va, A.va.data(), A.va.size(), s);
       if (e == cudaSuccess) e = silu::refill_slices(F->A->d, s);
-      if (e == cudaSuccess) e = upload_factors(F);
-      if (e == cudaSuccess) e = upload(F->d_dinv, F->dinv.data(), F->dinv.size(), s);
-      if (e == cudaSuccess && !F->dcol.empty()) e = upload(F->d_dcol, F->dcol.data(), F->dcol.size(), s);
+      if (e == cudaSuccess) e = with_room(ctx, [&] { return upload_solver(F); });
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);
       if (e != cudaSuccess) return cuda_err(ctx, e, "upload of the refactored factors");
       F->A->d.va = F->A->va.p;

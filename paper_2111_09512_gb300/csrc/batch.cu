@@ -313,6 +313,7 @@ __global__ void __launch_bounds__(KB) k_bdivide(int nch, const int4* __restrict_
 struct InnerGraph {
   int j = -1, mL = 0, mU = 0, precond = 0;
   int64_t gen = -1;  // launch configuration of the factors at capture
+  int64_t cgen = -1;  // and the context's copies
   cudaGraphExec_t exec = nullptr;
   int64_t kernels = 0;
 };
@@ -382,8 +383,7 @@ cudaError_t allocate_bkrylov(silu_batch B, int m) {
 }
 
 cudaError_t ensure_bkrylov(silu_batch B, int m) {
-  const cudaError_t e = allocate_bkrylov(B, m);
-  return e == cudaErrorMemoryAllocation && drop_slices(B->F) ? allocate_bkrylov(B, m) : e;
+  return with_room(B->ctx, [&] { return allocate_bkrylov(B, m); });
 }
 
 // The fixed kernel sequence of inner iteration j (on the batch's buffers).
@@ -435,7 +435,8 @@ void inner_iteration(silu_batch B, int j, int m, int mL, int mU, int precond, do
 void run_inner(silu_batch B, int j, int m, int mL, int mU, int precond, double tol, int maxit) {
   silu_ctx ctx = B->ctx;
   for (InnerGraph& ig : B->graphs)
-    if (ig.j == j && ig.mL == mL && ig.mU == mU && ig.precond == precond && ig.gen == B->F->config_gen) {
+    if (ig.j == j && ig.mL == mL && ig.mU == mU && ig.precond == precond && ig.gen == B->F->config_gen &&
+        ig.cgen == ctx->copies_gen) {
       ctx->launches += ig.kernels;
       CK(cudaGraphLaunch(ig.exec, ctx->stream));
       return;
@@ -468,6 +469,7 @@ void run_inner(silu_batch B, int j, int m, int mL, int mU, int precond, double t
   ig.mU = mU;
   ig.precond = precond;
   ig.gen = B->F->config_gen;
+  ig.cgen = ctx->copies_gen;
   ig.kernels = ctx->launches - l0;
   ctx->launches = l0;
   if (e == cudaSuccess) e = cudaGraphInstantiate(&ig.exec, graph, 0);
@@ -572,7 +574,8 @@ silu_status silu_batch_setup(silu_ctx ctx, int count, const int64_t* n, const in
         delete B;
         return ds;
       }
-      cudaError_t e = upload_csr(M->A, false, M->rp, M->ci, M->va, M->tiles, M->d, ctx->stream);
+      cudaError_t e =
+          with_room(ctx, [&] { return upload_csr(ctx, M->A, false, M->rp, M->ci, M->va, M->tiles, M->d); });
       if (e != cudaSuccess) {
         delete B;
         return cuda_err(ctx, e, "upload of the batch matrix");
@@ -596,8 +599,10 @@ silu_status silu_batch_setup(silu_ctx ctx, int count, const int64_t* n, const in
     }
     B->nch = (int)(B->chunks.size() / 4);
     if (ctx->device >= 0) {
-      cudaError_t e = upload(B->d_chunks, B->chunks.data(), B->chunks.size(), ctx->stream);
-      if (e == cudaSuccess) e = upload(B->d_sys_chunk0, B->sys_chunk0.data(), B->sys_chunk0.size(), ctx->stream);
+      cudaError_t e = with_room(ctx, [&] {
+        const cudaError_t u = upload(B->d_chunks, B->chunks.data(), B->chunks.size(), ctx->stream);
+        return u == cudaSuccess ? upload(B->d_sys_chunk0, B->sys_chunk0.data(), B->sys_chunk0.size(), ctx->stream) : u;
+      });
       if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
       if (e != cudaSuccess) {
         delete B;

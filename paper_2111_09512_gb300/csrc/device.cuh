@@ -51,6 +51,11 @@ constexpr int kTileNnzNarrow = 360;
 constexpr int kNarrowChunkRows = 10;
 constexpr double kNarrowMeanRow = 9.0;
 
+// Device memory of the library's objects, counted over the process, and
+// refused beyond the calling thread's limit (silu_selftest_memory).
+cudaError_t device_alloc(void** p, size_t bytes);
+void device_free(void* p, size_t bytes);
+
 // A matrix cut into slices of 32 consecutive rows, for k_slices (one warp per
 // slice, one lane per row; kernels_slices.cu).  Slice s holds, for k < width
 // (its longest row), entry k of every row, padded with value 0 and an
@@ -67,12 +72,14 @@ struct Slices {
   int2* hdr = nullptr;    // ns + 1 entries: {first slot, smallest column}
   void* ci = nullptr;     // uint16_t offsets, or int columns
   void* va = nullptr;     // double or float
-  void* buf = nullptr;    // the one allocation that holds the three
+  void* buf = nullptr;    // the one allocation that holds the three (null once given up, see drop_slices)
   size_t bytes = 0;       // and its size
+  bool sole = false;      // the CSR arrays are gone: this copy is not given up
+  void release();
   Slices() = default;
   Slices(const Slices&) = delete;
   Slices& operator=(const Slices&) = delete;
-  ~Slices();
+  ~Slices() { release(); }
 };
 
 struct DevCsr {
@@ -107,6 +114,7 @@ struct DevCsr {
   // the sliced copy (null: none); swept instead of the tiles unless a staged
   // launch shape was asked for (explicit_shape) or a sweep variant says so
   std::shared_ptr<Slices> sl;
+  bool sliced() const { return sl && sl->buf; }
   bool explicit_shape = false;
 };
 
@@ -211,7 +219,7 @@ bool staged_multi_ok(const DevCsr& T, int R);
 cudaError_t launch_sweep_staged_multi(const DevCsr& T, Mode mode, const LaunchEnv& env, int R, int ldx, const void* c,
                                       const void* in, void* out, const double* dinv, double* x, int epi,
                                       cudaStream_t s);
-// The sweep on the sliced copy T.sl for R = 1..4 interleaved right-hand sides
+// The sweep on the sliced copy (T.sliced()) for R = 1..4 interleaved right-hand sides
 // (leading dimension ldx >= R); with one column the bits of the tiled sweep
 // in its automatic shape.
 cudaError_t launch_sweep_slices(const DevCsr& T, Mode mode, const LaunchEnv& env, int R, int ldx, const void* c,

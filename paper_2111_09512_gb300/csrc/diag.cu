@@ -65,15 +65,16 @@ extern "C" silu_status silu_ilu_power_norms(silu_ilu F, int which, int pmax, int
     transpose(T, Tt);
     DBuf rp, ci, va, tiles, trp, tci, tva, ttiles, dv0, dv, da, db, part, dout, dz;
     DevCsr dT, dTt;
-    CK(silu::upload_csr(T, false, rp, ci, va, tiles, dT, s));
-    CK(silu::upload_csr(Tt, false, trp, tci, tva, ttiles, dTt, s));
-    CK(silu::upload(dv0, v0, (size_t)n, s));
-    CK(dv.ensure(sizeof(double) * n));
-    CK(da.ensure(sizeof(double) * n));
-    CK(db.ensure(sizeof(double) * n));
-    CK(part.ensure(sizeof(double) * 1024));
-    CK(dout.ensure(sizeof(double) * (size_t)pmax));
-    CK(dz.ensure(sizeof(double)));
+    CK(silu::with_room(ctx, [&] {
+      cudaError_t e = silu::upload_csr(ctx, T, false, rp, ci, va, tiles, dT);
+      if (e == cudaSuccess) e = silu::upload_csr(ctx, Tt, false, trp, tci, tva, ttiles, dTt);
+      if (e == cudaSuccess) e = silu::upload(dv0, v0, (size_t)n, s);
+      for (DBuf* d : {&dv, &da, &db})
+        if (e == cudaSuccess) e = d->ensure(sizeof(double) * n);
+      if (e == cudaSuccess) e = part.ensure(sizeof(double) * 1024);
+      if (e == cudaSuccess) e = dout.ensure(sizeof(double) * (size_t)pmax);
+      return e == cudaSuccess ? dz.ensure(sizeof(double)) : e;
+    }));
     double* v = dv.as<double>();
     double* a = da.as<double>();
     double* b = db.as<double>();

@@ -23,11 +23,6 @@
 
 namespace silu {
 
-// Device memory of the library's objects, counted over the process, and
-// refused beyond the calling thread's limit (silu_selftest_memory).
-cudaError_t device_alloc(void** p, size_t bytes);
-void device_free(void* p, size_t bytes);
-
 // Owning device buffer.
 struct DBuf {
   void* p = nullptr;
@@ -76,6 +71,12 @@ struct silu_ctx_s {
   int device = -1;
   Copies copies = Copies::kBoth;         // of matrices and hierarchy operators
   Copies factor_copies = Copies::kBoth;  // of sweep factors
+  // the sliced copies of this context's objects, which give way when memory
+  // runs out (with_room); copies_gen counts these occasions (captured graphs
+  // that sweep such copies go stale)
+  std::vector<std::weak_ptr<silu::Slices>> slices;
+  int64_t copies_gen = 0;
+  bool no_copies = false;  // build none: silu_ctx_set_copies, or memory ran out in the call that is under way
   cudaStream_t stream = nullptr;
   std::string err;
   double* pinned = nullptr;  // small host buffer for scalar read-backs
@@ -112,6 +113,7 @@ struct KrylovGraph {
   int j = -1, m = 0, mL = 0, mU = 0, precond = 0;
   int64_t gen = -1;   // launch configuration the graph was captured with
   int64_t agen = -1;  // and the matrix's
+  int64_t cgen = -1;  // and the context's copies
   cudaGraphExec_t exec = nullptr;
   int64_t kernels = 0;
 };
@@ -367,16 +369,32 @@ cudaError_t upload(DBuf& b, const T* src, size_t count, cudaStream_t s) {
 // Upload CSR (int64 row pointers narrowed to int32) with values as double or
 // float.  Arrays get kCsrPad spare (zeroed) elements for the staged kernel's
 
-cudaError_t upload_csr(const Csr& T, bool fp32, DBuf& rp, DBuf& ci, DBuf& va, DBuf& tiles, DevCsr& d,
-                       cudaStream_t s, Copies copies = Copies::kBoth);
-// Drop the sliced copies of F's factors and of A (false if there are none).
-bool drop_slices(silu_ilu F);
+cudaError_t upload_csr(silu_ctx ctx, const Csr& T, bool fp32, DBuf& rp, DBuf& ci, DBuf& va, DBuf& tiles, DevCsr& d,
+                       Copies copies = Copies::kBoth);
+// Give up the sliced copies of ctx's objects (false if there are none): their
+// sweeps run on the tiles, for one right-hand side with the same bits.
+bool drop_slices(silu_ctx ctx);
+// make(), which allocates, once more without sliced copies if memory ran out:
+// what a call needs comes before copies that only make sweeps faster.
+template <class Make>
+cudaError_t with_room(silu_ctx ctx, Make make) {
+  const cudaError_t e = make();
+  if (e != cudaErrorMemoryAllocation || !drop_slices(ctx)) return e;
+  cudaGetLastError();
+  struct Hold {
+    silu_ctx c;
+    bool was;
+    explicit Hold(silu_ctx x) : c(x), was(x->no_copies) { c->no_copies = true; }
+    ~Hold() { c->no_copies = was; }
+  } hold(ctx);
+  return make();
+}
 // The tile entry limit of the automatic launch shape: narrow tiles for FP64
 // values with one lane per row whose rows fit them (silu::narrow_fits).
 int auto_tile_nnz(const Csr& T, bool fp32, int lanes, int passes);
 // Length-sorted copy of T for the staged kernel (silu::make_sorted); clears
 // the copy in d when it would not pay.
-cudaError_t upload_sorted(const Csr& T, bool fp32, SortedBufs& b, DevCsr& d, cudaStream_t s);
+cudaError_t upload_sorted(silu_ctx ctx, const Csr& T, bool fp32, SortedBufs& b, DevCsr& d);
 // Upload L_s and the upper sweep factor of F with their sorted copies,
 // keeping the launch shapes chosen earlier (autotuner, variant).
 cudaError_t upload_factors(silu_ilu F);

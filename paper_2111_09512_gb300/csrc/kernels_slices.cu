@@ -8,8 +8,9 @@
 
 namespace silu {
 
-Slices::~Slices() {
-  if (buf) cudaFree(buf);
+void Slices::release() {
+  if (buf) device_free(buf, bytes);
+  buf = nullptr;
 }
 
 namespace {
@@ -206,7 +207,7 @@ cudaError_t build_slices(const int64_t* rp, DevCsr& d, cudaStream_t s) {
   const size_t vb = ((d.fp32 ? sizeof(float) : sizeof(double)) * slots + 255) / 256 * 256;
   auto allocate = [&](size_t col_bytes) {
     S->bytes = hb + vb + col_bytes * slots;
-    const cudaError_t e = cudaMalloc(&S->buf, S->bytes);
+    const cudaError_t e = device_alloc(&S->buf, S->bytes);
     S->hdr = (int2*)S->buf;
     S->va = (char*)S->buf + hb;
     S->ci = (char*)S->buf + hb + vb;
@@ -233,8 +234,7 @@ cudaError_t build_slices(const int64_t* rp, DevCsr& d, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     if (widest < 65535 || S->wide) break;  // offset 65535 marks padding
     S->wide = true;
-    cudaFree(S->buf);
-    S->buf = nullptr;
+    S->release();
     e = allocate(sizeof(int));
     if (e != cudaSuccess) return give_up(e);
   }
@@ -244,7 +244,7 @@ cudaError_t build_slices(const int64_t* rp, DevCsr& d, cudaStream_t s) {
 }
 
 cudaError_t refill_slices(const DevCsr& d, cudaStream_t s) {
-  if (!d.sl) return cudaSuccess;
+  if (!d.sliced()) return cudaSuccess;
   return d.fp32 ? fill<float>(d, *d.sl, s) : fill<double>(d, *d.sl, s);
 }
 
@@ -256,7 +256,7 @@ cudaError_t slices_prepare() {
 
 cudaError_t launch_sweep_slices(const DevCsr& T, Mode mode, const LaunchEnv& env, int R, int ldx, const void* c,
                                 const void* in, void* out, const double* dinv, double* x, int epi, cudaStream_t s) {
-  if (!T.sl || R < 1 || R > 4 || ldx < R || (R == 1 && ldx != 1)) return cudaErrorInvalidValue;
+  if (!T.sliced() || R < 1 || R > 4 || ldx < R || (R == 1 && ldx != 1)) return cudaErrorInvalidValue;
   if (R > 1) return launch_slices_multi(T, mode, env, R, ldx, c, in, out, dinv, x, epi, s);
   if (slices_ring_fits(T, mode, env.sms)) return launch_slices_ring(T, env, c, in, out, dinv, x, epi, s);
   const bool wide = T.sl->wide;

@@ -184,22 +184,25 @@ silu_status silu_schur_setup(silu_ilu F, int parts, double tau, int fill) {
       silu_status ds = silu::device_ok(ctx);
       if (ds != SILU_OK) return ds;
       cudaStream_t s = ctx->stream;
-      cudaError_t e = silu::ensure_vectors(S->FB, 1);
-      if (e == cudaSuccess) e = silu::upload_csr(E, false, S->E_rp, S->E_ci, S->E_va, S->E_t, S->E, s);
-      if (e == cudaSuccess) e = silu::upload_csr(Fm, false, S->F_rp, S->F_ci, S->F_va, S->F_t, S->F, s);
-      if (e == cudaSuccess) e = silu::upload_csr(C, false, S->C_rp, S->C_ci, S->C_va, S->C_t, S->C, s);
-      if (e == cudaSuccess) e = silu::upload(S->rowsI, rowsI.data(), rowsI.size(), s);
-      if (e == cudaSuccess) e = silu::upload(S->rowsG, rowsG.data(), rowsG.size(), s);
       const size_t bi = sizeof(double) * (size_t)std::max<int64_t>(S->nI, 1);
       const size_t bg = sizeof(double) * (size_t)std::max<int64_t>(S->nG, 1);
-      for (DBuf* d : {&S->f, &S->u, &S->t, &S->xi})
-        if (e == cudaSuccess) e = d->ensure(bi);
-      for (DBuf* d : {&S->g, &S->s, &S->w, &S->y, &S->q})
-        if (e == cudaSuccess) e = d->ensure(bg);
-      if (e == cudaSuccess && S->nG > 0) e = silu::upload(S->cdinv, cdinv.data(), cdinv.size(), s);
-      if (e == cudaSuccess) e = S->r.ensure(sizeof(double) * (size_t)std::max<int64_t>(n, 1));
-      if (e == cudaSuccess) e = S->part0.ensure(sizeof(double) * 1024);
-      if (e == cudaSuccess) e = S->part1.ensure(sizeof(double) * 1024);
+      cudaError_t e = silu::ensure_vectors(S->FB, 1);
+      if (e == cudaSuccess)
+        e = silu::with_room(ctx, [&] {
+          cudaError_t u = silu::upload_csr(ctx, E, false, S->E_rp, S->E_ci, S->E_va, S->E_t, S->E);
+          if (u == cudaSuccess) u = silu::upload_csr(ctx, Fm, false, S->F_rp, S->F_ci, S->F_va, S->F_t, S->F);
+          if (u == cudaSuccess) u = silu::upload_csr(ctx, C, false, S->C_rp, S->C_ci, S->C_va, S->C_t, S->C);
+          if (u == cudaSuccess) u = silu::upload(S->rowsI, rowsI.data(), rowsI.size(), s);
+          if (u == cudaSuccess) u = silu::upload(S->rowsG, rowsG.data(), rowsG.size(), s);
+          for (DBuf* d : {&S->f, &S->u, &S->t, &S->xi})
+            if (u == cudaSuccess) u = d->ensure(bi);
+          for (DBuf* d : {&S->g, &S->s, &S->w, &S->y, &S->q})
+            if (u == cudaSuccess) u = d->ensure(bg);
+          if (u == cudaSuccess && S->nG > 0) u = silu::upload(S->cdinv, cdinv.data(), cdinv.size(), s);
+          if (u == cudaSuccess) u = S->r.ensure(sizeof(double) * (size_t)std::max<int64_t>(n, 1));
+          if (u == cudaSuccess) u = S->part0.ensure(sizeof(double) * 1024);
+          return u == cudaSuccess ? S->part1.ensure(sizeof(double) * 1024) : u;
+        });
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);
       if (e != cudaSuccess) return silu::cuda_err(ctx, e, "upload of the Schur complement smoother");
     }

@@ -121,3 +121,109 @@ def test_tiles_stay_in_place_when_new_ones_do_not_fit(silu, limit):
     out_of_memory(silu, lambda: M.set_shape(4, 1, 16))
     M.residual(r, x, b)
     assert relerr(host(r), oracle.residual(A, host(x), host(b))) < FP64_TOL
+
+
+def every_setup(silu, ctx):
+    """One of each object and call that takes device memory, in one context; all results for one right-hand side."""
+    A = synth.cutcell7(*SHAPE, seed=2)
+    n = len(A[0]) - 1
+    b = dev(synth.rhs(n, 1, seed=6)[:, 0])
+    out, kept = [], []
+
+    def result(call):
+        x = torch.zeros_like(b)
+        call(x)
+        ctx.check()
+        out.append(host(x))
+
+    M = silu.Matrix(ctx, *A)
+    F = silu.ilu_setup(ctx, M, "ilu0")
+    out.append(F.power_norms("U", 2, 3, synth.rhs(n, 1, seed=7)[:, 0]))
+    F.set_direct(1)  # the automatic choice is timed
+    result(lambda x: silu.direct_trisolve(F, x, b))
+    result(lambda x: silu.ilu_smooth(F, x, b, 3, 3))
+    result(lambda x: silu.fgmres_solve(F, x, b, tol=0.0, restart=25, maxit=9, sweeps_L=2, sweeps_U=2))
+    F.amg_setup(coarse_size=100, ilu_levels=2)
+    result(lambda x: F.amg_vcycle(x, b, 2, 2))
+    F.schur_setup(3, 1e-3, 5)
+    result(lambda x: F.schur_smooth(x, b, 2, 2))
+    G = silu.ilu_setup(ctx, M, "ilut", 1e-3, 10, prec=silu.FP32)
+    G.set_direct(2)
+    result(lambda x: silu.ilu_smooth(G, x, b, 3, 3))
+    result(lambda x: silu.direct_trisolve(G, x, b))
+    result(lambda x: silu.fgmres_solve(F, x, b, tol=0.0, restart=25, maxit=9, sweeps_L=2, sweeps_U=2))
+    B = silu.Batch(ctx, [A, synth.cutcell7(9, 9, 9, seed=1)], "ilu0")
+    bb = dev(synth.rhs(B.n, 1, seed=8)[:, 0])
+    xb = torch.zeros_like(bb)
+    silu.silu_batch_fgmres(B, xb, bb, tol=0.0, restart=11, maxit=9, sweeps_L=2, sweeps_U=2)
+    ctx.check()
+    out.append(host(xb))
+    silu.ilu_refactor(F, A[2] * 2.0)
+    result(lambda x: silu.ilu_smooth(F, x, b, 3, 3))
+    kept += [M, F, G, B]
+    return out, kept
+
+
+def test_what_fits_without_sliced_copies_still_fits(silu, limit):
+    """Memory for the objects alone: the copies give way in every setup, and results keep their bits."""
+    base = silu.silu_selftest_memory()
+    ctx = silu.Context(0, torch.cuda.current_stream())
+    free, kept = every_setup(silu, ctx)
+    with_copies = silu.silu_selftest_memory() - base
+    del kept
+    ctx = silu.Context(0, torch.cuda.current_stream())
+    ctx.set_copies(False)
+    bare, kept = every_setup(silu, ctx)
+    without = silu.silu_selftest_memory() - base
+    assert without < with_copies
+    del kept
+    ctx = silu.Context(0, torch.cuda.current_stream())
+    limit(base + without)
+    short, kept = every_setup(silu, ctx)
+    for other in (bare, short):
+        assert len(other) == len(free)
+        assert all(np.array_equal(f, o) for f, o in zip(free, other))
+
+
+def test_a_workspace_takes_the_memory_of_the_copies(silu, limit):
+    """Growth of the workspace by as much as the copies hold, also after an exact solve, whose factors are those of
+    the sweeps."""
+    ctx = silu.Context(0, torch.cuda.current_stream())
+    A = synth.cutcell7(*SHAPE, seed=2)
+    n = len(A[0]) - 1
+    F = silu.ilu_setup(ctx, silu.Matrix(ctx, *A), "ilu0")
+    b = dev(synth.rhs(n, 1, seed=6)[:, 0])
+    x = torch.zeros_like(b)
+    silu.direct_trisolve(F, x, b)
+    F.reserve(1, 20)
+    torch.cuda.synchronize()
+    limit(silu.silu_selftest_memory())
+    # A and two factors, 13 entries a row: copies of at least 10 bytes an entry
+    F.reserve(3, 20)  # 4 vectors of 16 bytes a row more
+    F.reserve(3, 23)  # 48 bytes a row more
+
+
+def test_giving_up_the_copies_keeps_results_and_captured_solves(silu):
+    ctx = silu.Context(0, torch.cuda.current_stream())
+    A = synth.cutcell7(*SHAPE, seed=2)
+    n = len(A[0]) - 1
+    M = silu.Matrix(ctx, *A)
+    F = silu.ilu_setup(ctx, M, "ilu0")
+    B = silu.Batch(ctx, [A], "ilu0")
+    b = dev(synth.rhs(n, 1, seed=6)[:, 0])
+    out = []
+    for copies in (True, False):
+        ctx.set_copies(copies)
+        x, y, r = torch.zeros_like(b), torch.zeros_like(b), torch.zeros_like(b)
+        silu.fgmres_solve(F, x, b, tol=0.0, restart=7, maxit=9, sweeps_L=2, sweeps_U=2)
+        silu.silu_batch_fgmres(B, y, b, tol=0.0, restart=7, maxit=9, sweeps_L=2, sweeps_U=2)
+        M.residual(r, x, b)
+        ctx.check()
+        out.append((host(x), host(y), host(r)))
+    assert all(np.array_equal(p, q) for p, q in zip(*out))
+    used = silu.silu_selftest_memory()
+    M2 = silu.Matrix(ctx, *A)
+    bare = silu.silu_selftest_memory() - used
+    ctx.set_copies(True)
+    M3 = silu.Matrix(ctx, *A)
+    assert silu.silu_selftest_memory() - used > 2 * bare + 10 * 6 * n
