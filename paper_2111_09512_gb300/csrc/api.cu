@@ -68,7 +68,6 @@ cudaError_t upload_csr(silu_ctx ctx, const silu::Csr& T, bool fp32, DBuf& rp, DB
   d.va = va.p;
   d.fp32 = fp32;
   d.explicit_shape = false;
-  d.sl.reset();
   std::vector<int> tl;
   const int tlanes = silu::staged_lanes(T.rp.data(), T.n);
   const int tpasses = silu::staged_passes(T.rp.data(), T.n, tlanes);
@@ -81,17 +80,21 @@ cudaError_t upload_csr(silu_ctx ctx, const silu::Csr& T, bool fp32, DBuf& rp, DB
   d.tile_passes = tpasses;
   d.tile_nnz = tnnz;
   // the sliced copy last, in what memory the arrays above leave
-  const bool slice = copies != Copies::kCsr && !ctx->no_copies && silu::slices_pay(T.rp.data(), T.n, fp32);
-  if (e == cudaSuccess && slice) {
-    e = silu::build_slices(T.rp.data(), d, s);
-    if (e == cudaSuccess && d.sl) {
+  std::vector<int2> hdr;
+  bool synced = false;
+  if (e == cudaSuccess && copies != Copies::kCsr && !ctx->no_copies &&
+      silu::slices_pay(T.rp.data(), T.n, fp32, hdr)) {
+    const Slices* const had = d.sl.get();
+    e = silu::build_slices(hdr, tlanes, d, s);
+    synced = e == cudaSuccess && d.sl;
+    if (synced && d.sl.get() != had) {
       auto& all = ctx->slices;
       all.erase(std::remove_if(all.begin(), all.end(), [](const auto& w) { return w.expired(); }), all.end());
       all.push_back(d.sl);
     }
+  } else {
+    d.sl.reset();
   }
-  // host staging vectors die at return, and a sweep reads the matrix ahead of the kernel before it
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e == cudaSuccess && d.sl && copies == Copies::kSmaller) {
     if (tiled && d.sl->bytes > rp.bytes + ci.bytes + va.bytes + tiles.bytes) {
       d.sl.reset();

@@ -225,12 +225,14 @@ cudaError_t launch_sweep_staged_multi(const DevCsr& T, Mode mode, const LaunchEn
 cudaError_t launch_sweep_slices(const DevCsr& T, Mode mode, const LaunchEnv& env, int R, int ldx, const void* c,
                                 const void* in, void* out, const double* dinv, double* x, int epi, cudaStream_t s);
 // Whether a matrix with this row pointer gets a sliced copy (see the
-// definition for the limit on padding).
-bool slices_pay(const int64_t* rp, int64_t n, bool fp32);
-// Build d.sl on the device from d's uploaded CSR arrays (rp: the host row
-// pointer, for which slices_pay holds).  A failed allocation leaves d.sl null
-// and is not an error.  Blocks on s until the headers are copied.
-cudaError_t build_slices(const int64_t* rp, DevCsr& d, cudaStream_t s);
+// definition for the limit on padding); hdr: the slices' first slots, then the
+// number of all.
+bool slices_pay(const int64_t* rp, int64_t n, bool fp32, std::vector<int2>& hdr);
+// Build d.sl on the device from d's uploaded CSR arrays and the headers of
+// slices_pay, in the buffer of the copy that d has if it is as large.  A
+// failed allocation leaves d.sl null and is not an error.  Blocks on s until
+// all that was queued before it, the copy of the headers included, is done.
+cudaError_t build_slices(const std::vector<int2>& hdr, int lanes, DevCsr& d, cudaStream_t s);
 // New values on the same pattern: fill d.sl again from d's CSR arrays (on s).
 cudaError_t refill_slices(const DevCsr& d, cudaStream_t s);
 // Give the slice kernels' instantiations the whole L1 (once per context).

@@ -26,24 +26,6 @@ constexpr double kSlicePadMax = 1.4;
 constexpr double kSlicePadFree = 2048.0;
 constexpr int64_t kMaxSlots = (int64_t)INT32_MAX - 65536;  // slot numbers (and a chunk beyond the last) fit an int
 
-// The slots of all slices (their first slots into *hdr, the longest row of all into *widest).
-int64_t slice_widths(const int64_t* rp, int64_t n, std::vector<int2>* hdr, int* widest = nullptr) {
-  int64_t slots = 0, most = 0;
-  const int64_t ns = (n + 31) / 32;
-  if (hdr) hdr->resize((size_t)ns + 1);
-  for (int64_t s = 0; s < ns; ++s) {
-    if (hdr) (*hdr)[(size_t)s] = make_int2((int)slots, 0);
-    int64_t w = 0;
-    for (int64_t r = s * 32; r < std::min<int64_t>(n, s * 32 + 32); ++r) w = std::max<int64_t>(w, rp[r + 1] - rp[r]);
-    slots += 32 * w;
-    most = std::max(most, w);
-    if (slots > kMaxSlots) return slots;
-  }
-  if (hdr) (*hdr)[(size_t)ns] = make_int2((int)slots, 0);
-  if (widest) *widest = (int)most;
-  return slots;
-}
-
 // Smallest column of every slice into its header, largest span of any slice
 // into *span (at least 0).  One warp per slice.
 __global__ void k_slice_span(int ns, int n, const int* __restrict__ rp, const int* __restrict__ ci,
@@ -185,29 +167,49 @@ cudaError_t for_each_shape(F f) {
 
 }  // namespace
 
-bool slices_pay(const int64_t* rp, int64_t n, bool fp32) {
+bool slices_pay(const int64_t* rp, int64_t n, bool fp32, std::vector<int2>& hdr) {
+  hdr.clear();
   // FP32 rows of more than 16 entries on average keep the tiled sweep, whose
   // lanes share a row (an FP32 sum in another order differs by 1e-7)
   if (n <= 0 || (fp32 && staged_lanes(rp, n) > 1)) return false;
-  const int64_t slots = slice_widths(rp, n, nullptr);
-  return slots <= kMaxSlots && (double)slots <= kSlicePadMax * (double)rp[n] + kSlicePadFree;
+  const double most = std::min((double)kMaxSlots, kSlicePadMax * (double)rp[n] + kSlicePadFree);
+  const int64_t ns = (n + 31) / 32;
+  hdr.resize((size_t)ns + 1);
+  int64_t slots = 0;
+  for (int64_t s = 0; s < ns; ++s) {
+    hdr[(size_t)s] = make_int2((int)slots, 0);
+    int64_t w = 0;
+    for (int64_t r = s * 32; r < std::min<int64_t>(n, s * 32 + 32); ++r) w = std::max<int64_t>(w, rp[r + 1] - rp[r]);
+    slots += 32 * w;
+    if ((double)slots > most) return false;
+  }
+  hdr[(size_t)ns] = make_int2((int)slots, 0);
+  return true;
 }
 
-cudaError_t build_slices(const int64_t* rp, DevCsr& d, cudaStream_t s) {
-  d.sl.reset();
-  std::shared_ptr<Slices> S(new (std::nothrow) Slices);
+cudaError_t build_slices(const std::vector<int2>& hdr, int lanes, DevCsr& d, cudaStream_t s) {
+  std::shared_ptr<Slices> S;
+  S.swap(d.sl);
+  if (!S || S.use_count() > 1 || S->sole) S.reset(new (std::nothrow) Slices);
   if (!S) return cudaSuccess;
-  std::vector<int2> hdr;
-  S->slots = slice_widths(rp, d.n, &hdr, &S->widest);
+  S->slots = hdr.back().x;
   S->ns = (int)hdr.size() - 1;
-  S->lanes = staged_lanes(rp, d.n);
+  S->lanes = lanes;
+  S->wide = false;
+  S->widest = 0;
+  for (size_t k = 0; k + 1 < hdr.size(); ++k) S->widest = std::max(S->widest, (hdr[k + 1].x - hdr[k].x) / 32);
   // one allocation: the headers and, past them, one int for the span; values; columns
   const size_t hb = (sizeof(int2) * (hdr.size() + 1) + 255) / 256 * 256;
   const size_t slots = (size_t)std::max<int64_t>(S->slots, 32);
   const size_t vb = ((d.fp32 ? sizeof(float) : sizeof(double)) * slots + 255) / 256 * 256;
   auto allocate = [&](size_t col_bytes) {
-    S->bytes = hb + vb + col_bytes * slots;
-    const cudaError_t e = device_alloc(&S->buf, S->bytes);
+    const size_t bytes = hb + vb + col_bytes * slots;
+    cudaError_t e = cudaSuccess;
+    if (!S->buf || S->bytes != bytes) {  // else the buffer of the values before these
+      S->release();
+      e = device_alloc(&S->buf, bytes);
+    }
+    S->bytes = bytes;
     S->hdr = (int2*)S->buf;
     S->va = (char*)S->buf + hb;
     S->ci = (char*)S->buf + hb + vb;
@@ -230,15 +232,18 @@ cudaError_t build_slices(const int64_t* rp, DevCsr& d, cudaStream_t s) {
     e = cudaGetLastError();
     int widest = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&widest, span, sizeof(int), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // hdr is a host vector of this call
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return e;
     if (widest < 65535 || S->wide) break;  // offset 65535 marks padding
     S->wide = true;
-    S->release();
     e = allocate(sizeof(int));
     if (e != cudaSuccess) return give_up(e);
   }
   e = d.fp32 ? fill<float>(d, *S, s) : fill<double>(d, *S, s);
+  // A sweep reads the slices ahead of the wait for the kernel before it.  With
+  // an operation that is no kernel behind the fill, one that follows at once
+  // starts only when the fill is complete, without the host waiting for it.
+  if (e == cudaSuccess) e = cudaMemsetAsync(S->hdr + hdr.size(), 0, sizeof(int), s);
   if (e == cudaSuccess) d.sl = std::move(S);
   return e;
 }

@@ -227,3 +227,25 @@ def test_giving_up_the_copies_keeps_results_and_captured_solves(silu):
     ctx.set_copies(True)
     M3 = silu.Matrix(ctx, *A)
     assert silu.silu_selftest_memory() - used > 2 * bare + 10 * 6 * n
+
+
+@pytest.mark.parametrize("shape", [SHAPE, (258, 257, 2)], ids=["16-bit columns", "int32 columns"])
+def test_refactorisation_fills_the_copies_in_place(silu, limit, shape):
+    """New values on the same pattern take no memory, and the factors keep their sliced copies."""
+    ctx = silu.Context(0, torch.cuda.current_stream())
+    A, A2 = synth.cutcell7(*shape, seed=3), synth.cutcell7(*shape, seed=8)
+    n = len(A[0]) - 1
+    b, x0 = synth.rhs(n, 1, seed=5), synth.rhs(n, 1, seed=6)
+    for prec, tol in ((silu.FP64, FP64_TOL), (silu.FP32, 1e-5)):
+        F = silu.ilu_setup(ctx, silu.Matrix(ctx, *A), "ilu0", prec=prec)
+        F.reserve(1)
+        torch.cuda.synchronize()
+        used = silu.silu_selftest_memory()
+        limit(used)
+        silu.ilu_refactor(F, A2[2])
+        limit(-1)
+        assert silu.silu_selftest_memory() == used
+        x = dev(x0)
+        silu.ilu_smooth(F, x, dev(b), 4, 4)  # at once: the copies are complete when a sweep starts
+        S = oracle.row_scale(oracle.factor(A2, "ilu0", 0.0, 0))
+        assert relerr(host(x), oracle.smooth(A2, S, x0, b, 4, 4)) < tol
