@@ -437,7 +437,11 @@ void silu_ilu_destroy(silu_ilu F);
 /*
  * Kernel launch shape of the sweeps: lanes per row (power of two, 1..32) for
  * L_s, the upper factor and A; 0 restores the library's choice.  Used by the
- * autotuner; results do not depend on it beyond rounding order.
+ * autotuner; results do not depend on it beyond rounding order.  It is the
+ * shape of the lanes-per-row kernel: of variant 1 (silu_ilu_set_kernel), and
+ * in the automatic variant of two to four columns where neither the staged
+ * kernel nor the fused launch (silu_ilu_set_fused, mode 0) would take them,
+ * which then run on that kernel instead of the sliced one.
  */
 silu_status silu_ilu_set_lanes(silu_ilu F, int lanes_L, int lanes_U, int lanes_A);
 

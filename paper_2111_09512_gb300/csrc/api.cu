@@ -540,6 +540,9 @@ bool small_block(silu_ilu F, int R) {
 bool use_slices(silu_ilu F, const DevCsr& T, int R, int ldx) {
   if (!T.sliced() || T.explicit_shape || F->variant == 1 || R > 4 || (R == 1 && ldx != 1)) return false;
   if (F->variant != 0 && (&T == &F->dL || &T == &F->dU)) return false;
+  // lanes per row asked for (silu_ilu_set_lanes), where that kernel runs when there are no slices
+  const int lanes = &T == &F->dL ? F->lanesL : (&T == &F->dU ? F->lanesU : (&T == &F->A->d ? F->lanesA : 0));
+  if (lanes > 0 && T.rp && (R == 1 ? T.ntiles == 0 : !multi_tiles(F, T, R) && !small_block(F, R))) return false;
   // Large matrices that the tiled sweeps serve faster (per sweep, slices
   // against tiles):
   // - FP32, one column, int32 columns (no fewer bytes than the tiles, and no

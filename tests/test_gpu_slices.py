@@ -202,3 +202,25 @@ def test_long_rows_and_int32_columns_match_the_lanes_per_row_kernel(silu, ctx, g
                 ctx.check()
                 out.append(host(x))
             assert max(relerr(out[0][:, k], out[1][:, k]) for k in range(nrhs)) < tol, (prec, nrhs)
+
+
+def test_lanes_asked_for_are_used(silu, ctx):
+    """silu_ilu_set_lanes shapes the sweeps of several columns of the automatic variant: the bits of variant 1, not
+    those of the sliced sweeps (an eight-lane sum of up to 10 terms rounds differently in some row)."""
+    A = synth.cutcell7(21, 19, 17, seed=2)
+    n = len(A[0]) - 1
+    for prec in (silu.FP64, silu.FP32):
+        F = silu.ilu_setup(ctx, silu.Matrix(ctx, *A), "ilut", 1e-3, 10, prec=prec)
+        F.set_fused(1)
+        for nrhs in (2, 3, 4):
+            b, x0 = synth.rhs(n, nrhs, seed=5), synth.rhs(n, nrhs, seed=6)
+            out = {}
+            for variant, lanes in ((0, 0), (0, 8), (1, 8)):
+                F.set_kernel(variant)
+                F.set_lanes(lanes, lanes, lanes)
+                x = dev(x0)
+                silu.ilu_smooth(F, x, dev(b), 4, 4)
+                out[variant, lanes] = host(x)[:, :nrhs // 2 * 2]  # a third column goes by itself, on tiles or slices
+            assert np.array_equal(out[0, 8], out[1, 8]), (prec, nrhs)
+            if prec == silu.FP64:
+                assert not np.array_equal(out[0, 8], out[0, 0]), nrhs
