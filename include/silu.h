@@ -229,8 +229,9 @@ silu_status silu_mat_create(silu_ctx ctx, int64_t n, int64_t nnz, const int64_t*
 void silu_mat_destroy(silu_mat A);
 
 /*
- * Launch shape of the staged kernel on A (the residual r = b - A x and the
- * FGMRES products): lanes per row (0 = from the mean row length, else 1, 2
+ * Launch shape of the staged kernel on A for one right-hand side (the
+ * residual r = b - A x and the FGMRES products; several right-hand sides
+ * keep the library's choice of kernel): lanes per row (0 = from the mean row length, else 1, 2
  * or 4), rows per lane (0 = automatic, else 1, 2 or 4; more than one only
  * with one lane per row), gather width (8 or 16 entries in flight per lane;
  * 10: the narrow configuration -- tiles of at most 352 entries swept by 24

@@ -534,11 +534,11 @@ bool small_block(silu_ilu F, int R) {
 }
 
 // Whether a launch on T takes the sliced copy: the default wherever there is
-// one.  An explicit staged shape of A (silu_mat_set_shape) and, for the
-// factors, an explicit staged variant (2, 3) keep the tiles; variant 1 keeps
-// the lanes-per-row kernel everywhere.
+// one.  An explicit staged shape of A (silu_mat_set_shape, for one column)
+// and, for the factors, an explicit staged variant (2, 3) keep the tiles;
+// variant 1 keeps the lanes-per-row kernel everywhere.
 bool use_slices(silu_ilu F, const DevCsr& T, int R, int ldx) {
-  if (!T.sliced() || T.explicit_shape || F->variant == 1 || R > 4 || (R == 1 && ldx != 1)) return false;
+  if (!T.sliced() || (T.explicit_shape && R == 1) || F->variant == 1 || R > 4 || (R == 1 && ldx != 1)) return false;
   if (F->variant != 0 && (&T == &F->dL || &T == &F->dU)) return false;
   // lanes per row asked for (silu_ilu_set_lanes), where that kernel runs when there are no slices
   const int lanes = &T == &F->dL ? F->lanesL : (&T == &F->dU ? F->lanesU : (&T == &F->A->d ? F->lanesA : 0));
@@ -1574,7 +1574,7 @@ silu_status silu_mat_residual(silu_mat A, double* r, const double* x, const doub
   if (A->A.n == 0) return SILU_OK;
   cudaStream_t s = ctx->stream;
   try {
-    if (A->d.sliced() && !A->d.explicit_shape) {
+    if (A->d.sliced() && (nrhs > 1 || !A->d.explicit_shape)) {
       for (int c0 = 0; c0 < nrhs;) {
         const int w = slice_width(nrhs - c0);
         LAUNCH(ctx, SILU_K_RESIDUAL, silu::launch_sweep_slices(A->d, silu::MODE_D, ctx->env, w, nrhs, b + c0, x + c0,

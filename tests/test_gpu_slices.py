@@ -224,3 +224,22 @@ def test_lanes_asked_for_are_used(silu, ctx):
             assert np.array_equal(out[0, 8], out[1, 8]), (prec, nrhs)
             if prec == silu.FP64:
                 assert not np.array_equal(out[0, 8], out[0, 0]), nrhs
+
+
+def test_a_shape_for_one_column_leaves_several_columns_alone(silu, ctx):
+    """silu_mat_set_shape and its autotuner time one column; blocks of columns keep the sliced kernel's bits."""
+    A = synth.cutcell7(21, 19, 17, seed=2)
+    n = len(A[0]) - 1
+    M = silu.Matrix(ctx, *A)
+    F = silu.ilu_setup(ctx, M, "ilu0")
+    F.set_fused(1)
+    for nrhs in (2, 3, 4, 5):
+        b, x0 = synth.rhs(n, nrhs, seed=5), synth.rhs(n, nrhs, seed=6)
+        out = []
+        for shape in ((0, 0, 0), (4, 1, 16), (1, 2, 16)):
+            M.set_shape(*shape)
+            r, x = dev(np.zeros((n, nrhs))), dev(x0)
+            M.residual(r, x, dev(b))
+            silu.ilu_smooth(F, x, dev(b), 3, 3)
+            out.append((host(r), host(x)))
+        assert all(np.array_equal(p, q) for o in out[1:] for p, q in zip(out[0], o)), nrhs
