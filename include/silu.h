@@ -212,6 +212,12 @@ silu_status silu_ctx_selftest_timeout(silu_ctx ctx, int timeout_ms);
  * bytes (negative: no limit).  *in_use (may be NULL): that memory now.
  */
 silu_status silu_selftest_memory(int64_t limit, int64_t* in_use);
+/*
+ * Self-test of the division that normalises Krylov vectors (one divisor for
+ * many entries): q[i] = w[i] / h[i], correctly rounded, on n device entries.
+ * Asynchronous.
+ */
+silu_status silu_ctx_selftest_divide(silu_ctx ctx, int64_t n, const double* w, const double* h, double* q);
 /* Message of the last failed call on ctx ("" if none); valid until the next call. */
 const char* silu_last_error(silu_ctx ctx);
 /* Library version string. */

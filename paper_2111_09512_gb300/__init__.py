@@ -126,6 +126,7 @@ def load():
         "silu_ctx_check": (i32, [vp]),
         "silu_ctx_selftest_timeout": (i32, [vp, i32]),
         "silu_ilu_selftest_exchange": (i32, [vp]),
+        "silu_ctx_selftest_divide": (i32, [vp, i64, vp, vp, vp]),
         "silu_ctx_set_copies": (i32, [vp, i32]),
         "silu_selftest_memory": (i32, [i64, ctypes.POINTER(i64)]),
         "silu_ilu_set_kernel": (i32, [vp, i32]),
@@ -168,7 +169,7 @@ def exported_symbols():
             "silu_amg_level_ilu", "silu_amg_stats", "silu_amg_export_level", "silu_schur_setup", "silu_schur_smooth",
             "silu_schur_stats", "silu_schur_set_interface_prec",
             "silu_ilu_destroy", "silu_ilu_set_lanes", "silu_ctx_profile", "silu_ctx_profile_read",
-            "silu_ctx_launch_count", "silu_ctx_check", "silu_ctx_selftest_timeout", "silu_ilu_selftest_exchange", "silu_selftest_memory", "silu_ctx_set_copies", "silu_ilu_set_kernel", "silu_ilu_set_direct", "silu_ilu_set_fused", "silu_ilu_layout", "silu_ilu_tune_table", "silu_ctx_set_overlap",
+            "silu_ctx_launch_count", "silu_ctx_check", "silu_ctx_selftest_timeout", "silu_ilu_selftest_exchange", "silu_selftest_memory", "silu_ctx_selftest_divide", "silu_ctx_set_copies", "silu_ilu_set_kernel", "silu_ilu_set_direct", "silu_ilu_set_fused", "silu_ilu_layout", "silu_ilu_tune_table", "silu_ctx_set_overlap",
             "silu_ctx_set_l2_reuse",
             "silu_smooth_noalloc",
             "silu_batch_setup", "silu_batch_info", "silu_batch_smooth", "silu_batch_fgmres", "silu_batch_destroy",
@@ -255,6 +256,11 @@ class Context:
     def selftest_timeout(self, timeout_ms: int = 50):
         """Run a bounded GPU wait on a flag nothing sets (the next check() reports ERR_TIMEOUT)."""
         _check(self.handle, load().silu_ctx_selftest_timeout(self.handle, timeout_ms), "silu_ctx_selftest_timeout")
+
+    def selftest_divide(self, w, h, q):
+        """q = w / h on device vectors by the division that normalises Krylov vectors."""
+        _check(self.handle, load().silu_ctx_selftest_divide(self.handle, w.numel(), _ptr(w), _ptr(h), _ptr(q)),
+               "silu_ctx_selftest_divide")
 
     def launch_count(self) -> int:
         """Kernels this context has launched since it was created."""

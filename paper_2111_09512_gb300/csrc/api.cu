@@ -1364,6 +1364,18 @@ silu_status silu_selftest_memory(int64_t limit, int64_t* in_use) {
   return SILU_OK;
 }
 
+silu_status silu_ctx_selftest_divide(silu_ctx ctx, int64_t n, const double* w, const double* h, double* q) {
+  if (!ctx || n < 0 || (n > 0 && (!w || !h || !q))) return SILU_ERR_INVALID_ARG;
+  silu_status ds = device_ok(ctx);
+  if (ds != SILU_OK) return ds;
+  try {
+    LAUNCH(ctx, SILU_K_KRYLOV, silu::launch_divide(n, w, h, q, ctx->stream));
+  } catch (const CudaFail& f) {
+    return cuda_err(ctx, f.e, f.what);
+  }
+  return SILU_OK;
+}
+
 silu_status silu_ilu_selftest_exchange(silu_ilu F) {
   if (!F) return SILU_ERR_INVALID_ARG;
   silu_ctx ctx = F->ctx;

@@ -63,10 +63,12 @@ __device__ __forceinline__ void collect(const ulonglong2* e, int stride, int cnt
 
 // w / h for many w: correctly rounded, five FP64 operations instead of the
 // division's twelve or so (which made normalising 1.9 M rows 48 us of FP64
-// work).  r = RN(1/h); q0 = RN(w r); each step q + RN(w - q h) r is an FMA on
-// an exact remainder: the first makes q faithful, the second correctly rounded
-// (Markstein, "IA-64 and Elementary Functions", Sec. 8.1: a correctly rounded
-// reciprocal and a faithful quotient give the rounded one).  That holds while
+// work).  r = RN(1/h); q0 = RN(w r), within two units in the last place; the
+// first step q + RN(w - q h) r makes q faithful, whatever its remainder loses
+// to rounding; the second starts from a faithful q, whose remainder an FMA
+// gives exactly, and rounds correctly (Markstein, "IA-64 and Elementary
+// Functions", Sec. 8.1: a correctly rounded reciprocal and a faithful quotient
+// give the rounded one).  That holds while
 // nothing over- or underflows, so operands outside the middle of the exponent
 // range (zeros, infinities and NaN among them) are divided.
 struct Divider {

@@ -203,6 +203,13 @@ __global__ void k_norm_final(const double* __restrict__ part_in, int nparts, dou
   if (threadIdx.x == 0) *out = h;
 }
 
+// q = w / h entry by entry, by the division the normalisations use.
+__global__ void k_divide(int64_t n, const double* __restrict__ w, const double* __restrict__ h,
+                         double* __restrict__ q) {
+  const int64_t i = blockIdx.x * (int64_t)KB + threadIdx.x;
+  if (i < n) q[i] = Divider(h[i])(w[i]);
+}
+
 // Every block solves the small triangle (redundantly, same order) and then
 // updates its slice of x with the combination of the preconditioned vectors.
 __global__ void __launch_bounds__(KB) k_update_x(int n, int jend, int m, const double* __restrict__ H,
@@ -275,6 +282,12 @@ cudaError_t launch_mr_step(int n, const double* part_num, const double* part_den
 
 cudaError_t launch_norm_final(int n, const double* part_in, double* out, cudaStream_t s) {
   k_norm_final<<<1, KB, 0, s>>>(part_in, krylov_parts(n), out);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_divide(int64_t n, const double* w, const double* h, double* q, cudaStream_t s) {
+  if (n <= 0) return cudaSuccess;
+  k_divide<<<(unsigned)((n + KB - 1) / KB), KB, 0, s>>>(n, w, h, q);
   return cudaGetLastError();
 }
 

@@ -31,6 +31,8 @@ cudaError_t launch_update_x(int n, int jend, int m, const double* H, const doubl
 // partial arrays written by launch_dot_part over n rows
 cudaError_t launch_mr_step(int n, const double* part_num, const double* part_den, const double* sv, double* y,
                            cudaStream_t s);
+// q = w / h entry by entry, by the normalisations' division (a self-test).
+cudaError_t launch_divide(int64_t n, const double* w, const double* h, double* q, cudaStream_t s);
 // One Arnoldi step in one launch (kernels_arnoldi.cu): w against columns 0..j
 // of V (stride n) by modified Gram-Schmidt, column j of H, V_{j+1} and the
 // Givens update, with the bits of launch_dot_part, launch_mgs_step,

@@ -157,3 +157,48 @@ def test_solve_after_a_step_that_gave_up(silu, size):
         assert st == silu.ERR_NOT_CONVERGED and its == 12
         out.append(x)
     assert torch.equal(out[0], out[1]) and torch.equal(out[0], out[2])
+
+
+def division_operands():
+    """(w, h): mantissas at random, all ones, next to powers of two and of few bits, with exponents on both sides of
+    the limits of the short division (2^+-300 of the divisor, 2^+-600 of the dividend), and the special values."""
+    rng = np.random.RandomState(5)
+
+    def mantissas(count):
+        m = rng.randint(0, 2**52, count, dtype=np.int64)
+        kind = rng.randint(0, 6, count)
+        m[kind == 1] = 2**52 - 1 - rng.randint(0, 4, (kind == 1).sum())
+        m[kind == 2] = rng.randint(0, 4, (kind == 2).sum())
+        m[kind == 3] &= -(1 << 40)
+        return m
+
+    def doubles(m, e):
+        return ((np.asarray(e, np.int64) + 1023 << 52) | m | (rng.randint(0, 2, len(m)).astype(np.int64) << 63)).view(
+            np.float64)
+
+    n = 1 << 21
+    out = [(doubles(mantissas(n), rng.randint(-40, 41, n)), doubles(mantissas(n), rng.randint(-40, 41, n)))]
+    edge_w, edge_h = np.array([-601, -600, -599, 598, 599, 600, 601]), np.array([-301, -300, -299, 298, 299, 300, 301])
+    out.append((doubles(mantissas(n), rng.choice(edge_w, n)), doubles(mantissas(n), rng.choice(edge_h, n))))
+    out.append((doubles(mantissas(n), rng.randint(-1022, 1024, n)), doubles(mantissas(n), rng.randint(-1022, 1024, n))))
+    special = np.array([0.0, -0.0, 5e-324, -5e-324, 2.2250738585072009e-308, 2.2250738585072014e-308, 1.0, -3.0, 1e308,
+                        1.7976931348623157e308, np.inf, -np.inf, np.nan])
+    special = np.concatenate([special, doubles(mantissas(40), rng.randint(-1022, 1024, 40))])
+    w, h = np.meshgrid(special, special)
+    out.append((w.ravel(), h.ravel()))
+    return out
+
+
+def test_division_of_the_normalisation_is_correctly_rounded(silu):
+    ctx = silu.Context(0, torch.cuda.current_stream())
+    for w, h in division_operands():
+        wd, hd = torch.from_numpy(w.copy()).cuda(), torch.from_numpy(h.copy()).cuda()
+        q = torch.empty_like(wd)
+        ctx.selftest_divide(wd, hd, q)
+        ctx.check()
+        with np.errstate(all="ignore"):
+            want = w / h
+        got = q.cpu().numpy()
+        nan = np.isnan(want)
+        assert np.isnan(got[nan]).all()
+        assert np.array_equal(got[~nan].view(np.int64), want[~nan].view(np.int64))

@@ -243,3 +243,58 @@ def test_a_shape_for_one_column_leaves_several_columns_alone(silu, ctx):
             silu.ilu_smooth(F, x, dev(b), 3, 3)
             out.append((host(r), host(x)))
         assert all(np.array_equal(p, q) for o in out[1:] for p, q in zip(out[0], o)), nrhs
+
+
+# FP32 factors of at least 64 slices of 32 rows per SM: units of four, two and one slices, several units per warp
+# (stages are used again), the last unit and the last slice not full
+RING = [("ilu0", "cutcell7", (111, 109, 107), 0, 4), ("iluk", "cutcell7", (91, 89, 85), 1, 2),
+        ("ilu0", "hex27", (80, 71, 59), 0, 1)]
+
+
+@pytest.mark.parametrize("kind,gen,size,fill,unit", RING, ids=["4 slices", "2 slices", "1 slice"])
+def test_large_fp32_sweeps_through_the_ring(silu, ctx, kind, gen, size, fill, unit):
+    """One lane sums a row in column order in the ring as on tiles: the same bits; the oracle to the rounding of
+    FP32 factors (nine sweeps of up to 13 terms, 1e-5)."""
+    A = getattr(synth, gen)(*size, seed=4)
+    n = len(A[0]) - 1
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    slices = -(-n // 32)
+    assert n % 32 and slices >= 64 * sms and slices > 2 * unit * 32 * sms and (unit == 1 or slices % unit)
+    F = silu.ilu_setup(ctx, silu.Matrix(ctx, *A), kind, 0.0, fill, prec=silu.FP32)
+    L, U = F.export()["L"], F.export()["Us"]
+    longest = max(int(np.diff(L[0]).max()), int(np.diff(U[0]).max()))
+    assert {4: 0, 2: 4, 1: 8}[unit] < longest <= {4: 4, 2: 8, 1: 16}[unit]
+    b, x0 = synth.rhs(n, 1, seed=1), synth.rhs(n, 1, seed=2)
+    out = []
+    for variant in (0, 2):
+        F.set_kernel(variant)
+        x = dev(x0)
+        silu.ilu_smooth(F, x, dev(b), 5, 6)
+        ctx.check()
+        out.append(host(x))
+    assert np.array_equal(out[0], out[1])
+    S = oracle.row_scale(oracle.factor(A, kind, 0.0, fill))
+    assert relerr(out[0], oracle.smooth(A, S, x0, b, 5, 6)) < 1e-5
+
+
+@pytest.mark.parametrize("span", [65534, 65535], ids=["widest 16-bit", "narrowest int32"])
+def test_columns_at_the_limit_of_16_bits(silu, ctx, span):
+    """A slice of 32 rows coupled `up` and `down` rows away spans up + down + 31 columns."""
+    n, up = 65800, 32752
+    down = span - 31 - up
+    i = np.arange(n)
+    r = np.concatenate([i, i[:-up], i[down:]])
+    c = np.concatenate([i, i[up:], i[:-down]])
+    order = np.lexsort((c, r))
+    r, c = r[order], c[order]
+    rp = np.zeros(n + 1, np.int64)
+    np.add.at(rp, r + 1, 1)
+    A = np.cumsum(rp), c.astype(np.int32), np.where(r == c, 4.0, -synth.uniform(5, 1, len(r), 0.1, 1.0))
+    lo, hi = np.minimum.reduceat(c, A[0][:-1:32]), np.maximum.reduceat(c, A[0][:-1:32])
+    assert (hi - lo).max() == span
+    M = silu.Matrix(ctx, *A)
+    for nrhs in (1, 2, 3, 4):
+        b, x = synth.rhs(n, nrhs, seed=21), synth.rhs(n, nrhs, seed=22)
+        out = dev(np.zeros((n, nrhs)))
+        M.residual(out, dev(x), dev(b))
+        assert maxabs_err(host(out), oracle.residual(A, x, b)) < FP64_TOL, nrhs
