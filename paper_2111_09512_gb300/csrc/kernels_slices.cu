@@ -157,7 +157,7 @@ cudaError_t for_each_shape(F f) {
   add(f(Double1<float, int, 4>()));
   add(each_small<F, double>(f));
   add(each_small<F, float>(f));
-  add(f(SliceKernel<float, float, float, uint16_t, 1, 2, 6, false>()));
+  add(f(SliceKernel<float, float, float, uint16_t, 1, 2, 5, false>()));
   add(f(SliceKernel<float, float, float, uint16_t, 1, 4, 3, false>()));
   add(f(SliceKernel<float, float, float, uint16_t, 1, 7, 3, false>()));
   add(f(SliceKernel<float, float, float, int, 1, 2, 5, false>()));
@@ -266,8 +266,11 @@ cudaError_t launch_sweep_slices(const DevCsr& T, Mode mode, const LaunchEnv& env
   if (slices_ring_fits(T, mode, env.sms)) return launch_slices_ring(T, env, c, in, out, dinv, x, epi, s);
   const bool wide = T.sl->wide;
   const bool small = !wide && slice_small(T.sl->ns, env.sms);
-  // FP32, which only small matrices reach: a whole row per chunk where rows
-  // allow (27-point 32^3 4.5 us a sweep).
+  // FP32, where the ring does not fit (fewer slices, longer rows, int32
+  // columns): a whole row per chunk where rows allow (27-point 32^3 4.5 us a
+  // sweep).  Rows of up to four entries at 40 warps per SM and 48 registers:
+  // 48 warps spill (cut-cell 50^3 / 54^3 / 58^3 / 64^3 5+5 applications 25.0 /
+  // 26.1 / 26.5 / 34.2 us that way, 23.8 / 24.3 / 26.6 / 34.6 this way).
   const double mean = (double)T.sl->slots / (32.0 * (double)T.sl->ns);
   auto go = [&](auto k) { return decltype(k)::launch(T, env, ldx, c, in, out, dinv, x, epi, s); };
   switch (mode) {
@@ -282,7 +285,7 @@ cudaError_t launch_sweep_slices(const DevCsr& T, Mode mode, const LaunchEnv& env
     case MODE_F:
       if (mean <= 4.0 && !(small && T.sl->widest > 4))
         return wide ? go(SliceKernel<float, float, float, int, 1, 2, 5, false>())
-                    : go(SliceKernel<float, float, float, uint16_t, 1, 2, 6, false>());
+                    : go(SliceKernel<float, float, float, uint16_t, 1, 2, 5, false>());
       if (wide || mean <= 8.0 || mean > 14.0)
         return wide ? go(SliceKernel<float, float, float, int, 1, 4, 3, false>())
                     : go(SliceKernel<float, float, float, uint16_t, 1, 4, 3, false>());

@@ -51,3 +51,30 @@ def test_sweep_blocks_fit_the_register_file(reports):
         args = name.split("k_sweep_rowsI", 1)[1]
         warps = int(args.split("ELi")[1])
         assert warps * 32 * regs <= 65536, (name, warps, regs)
+
+
+@pytest.fixture(scope="module")
+def all_reports(reports):
+    if not all(os.path.exists(os.path.join(_build.BUILD, u + ".ptxas.txt")) for u in _build.CU_SOURCES):
+        _build.build(force=True)
+    return {u: _build.kernel_resources(u) for u in _build.CU_SOURCES}
+
+
+def test_no_kernel_of_any_unit_spills(all_reports):
+    """The sliced sweeps, the one-launch Arnoldi step and the batch's kernels among them."""
+    for unit in ("kernels_slices.cu", "kernels_slices_multi.cu", "kernels_slices_ring.cu", "kernels_arnoldi.cu",
+                 "batch.cu"):
+        assert all_reports[unit], unit
+    spilling = {(u, k): v for u, kernels in all_reports.items() for k, v in kernels.items() if v[1] or v[2]}
+    assert not spilling, spilling
+
+
+def test_large_blocks_fit_the_register_file(all_reports):
+    """The ring's 32 warps and the Arnoldi step's one to three groups of eight, one block per SM."""
+    ring = {k: v for k, v in all_reports["kernels_slices_ring.cu"].items() if "k_slices_ring" in k}
+    groups = {k: v for k, v in all_reports["kernels_arnoldi.cu"].items() if "k_arnoldiILi" in k}
+    assert len(ring) == 3 and len(groups) == 3
+    assert all(1024 * regs <= 65536 for regs, _, _ in ring.values()), ring
+    for name, (regs, _, _) in groups.items():
+        g = int(name.split("k_arnoldiILi")[1].split("E")[0])
+        assert g * 256 * (-(-regs // 8) * 8) <= 65536, (name, regs)
