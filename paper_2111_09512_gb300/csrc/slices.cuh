@@ -146,9 +146,9 @@ constexpr unsigned kEpiDinv = 1u << EPI_SCALE | 1u << EPI_SCALE_ADDX | 1u << EPI
                               1u << EPI_JAC_ADDX | 1u << EPI_JAC_SETX;
 constexpr unsigned kEpiX = 1u << EPI_ADDX | 1u << EPI_SCALE_ADDX | 1u << EPI_JAC_ADDX | 1u << EPI_RICH_ADDX;
 
-// Launch flag of small matrices, beside the L2 flags: block b of B walks the
-// slices [b ns / B, (b + 1) ns / B) (ns and B are small) instead of every
-// (B W)-th group of W.
+// Launch flag beside the L2 flags: block b of B walks the slices
+// [b ns / B, (b + 1) ns / B) (of few per warp: B ns fits 32 bits) instead of
+// every (B W)-th group of W.
 constexpr int kFlagSpread = 8;
 
 // CP pairs of entries per chunk, at least MINB blocks of (up to) 8 warps per SM,
@@ -317,14 +317,28 @@ __global__ void __launch_bounds__(kSliceThreads, MINB)
 constexpr int kSliceSmall = 16;
 inline bool slice_small(int ns, int sms) { return ns <= kSliceSmall * sms; }
 
+// Large matrices: every (B W)-th group of W slices to a block, all blocks
+// resident, so that neighbouring slices are swept at the same time.  In the
+// second and third round of the warps this leaves SMs of unequal loads where
+// a round is partly full (5+5 applications, 7-point ILU(0), rounds / us with
+// the slices dealt evenly: one column at 64^3 1.12 / 41.4 (45.6), 67^3 1.29 /
+// 47.3 (48.1), 70^3 1.47 / 56.2 (48.8), 73^3 1.67 / 57.5 (51.9), 86^3 2.73 /
+// 76.9 (73.4), 90^3 3.12 / 82 (90); two columns at 64^3 1.35 / 80.4 (70.8),
+// 73^3 2.00 / 91.6 (92.5)), so the slices are dealt evenly from 0.3 of a round.
+// Not with int32 columns, whose far gathers want all blocks in one window of
+// the vector (27-point 260 x 260 x 4 FP32 2.32 / 68 us (80)).
+constexpr double kSliceUneven = 0.3, kSliceFull = 0.97;
+
 struct SlicePlan {
   int warps, blocks, flags;
 };
-inline SlicePlan slice_plan(int ns, int sms, int most) {
+inline SlicePlan slice_plan(int ns, int sms, int most, bool wide) {
   constexpr int W = kSliceThreads / 32;
   if (!slice_small(ns, sms)) {
-    const int want = (ns + W - 1) / W;
-    return {W, want < sms * most ? want : sms * most, 0};
+    const int want = (ns + W - 1) / W, grid = want < sms * most ? want : sms * most;
+    const double rounds = (double)ns / (sms * most * W), last = rounds - (int)rounds;
+    const bool even = !wide && rounds > 1 && rounds < 3 && last >= kSliceUneven && last < kSliceFull;
+    return {W, grid, even ? kFlagSpread : 0};
   }
   const int full = ns > W * sms && most > 1 ? 2 * sms : sms;
   const int blocks = ns < full ? ns : full, share = (ns + blocks - 1) / blocks;
@@ -342,7 +356,7 @@ struct SliceKernel {
                             const double* dinv, double* x, int epi, cudaStream_t s) {
     const Slices& S = *T.sl;
     if (S.ns == 0) return cudaSuccess;
-    const SlicePlan plan = slice_plan(S.ns, env.sms, MINB);
+    const SlicePlan plan = slice_plan(S.ns, env.sms, MINB, sizeof(CT) == 4);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)plan.blocks);
     cfg.blockDim = dim3((unsigned)(plan.warps * 32));
