@@ -533,6 +533,52 @@ bool small_block(silu_ilu F, int R) {
   return F->fused_mode == 0 && scaled_upper(F) && (R == 2 || R == 4) && F->F.L.n <= kFusedMaxRows;
 }
 
+// Large matrices that the tiled sweeps serve faster than the slices (multi:
+// R > 1 columns would take the tiles).  A kernel's warps walk their tiles,
+// slices or units in rounds of one per warp, and where the rounds of one kernel
+// are full and the last one of the other is nearly empty, the first is ahead.
+// Times are 5+5 applications, slices against tiles, unless per sweep.
+bool tiles_faster(const DevCsr& T, int R, bool multi, const silu::LaunchEnv& env) {
+  const Slices& S = *T.sl;
+  const double per_warp = 1.0 / env.sms;
+  const double tiles = T.ntiles * per_warp / silu::tile_warps(T.fp32);
+  auto filled = [](double rounds) { return rounds / std::ceil(rounds); };
+  if (R == 1) {
+    if (T.ntiles == 0) return false;
+    if (T.fp32 && S.ns >= 64 * env.sms) {
+      // int32 columns (no fewer bytes than the tiles, and no ring): 27-point 260
+      // x 260 x 30 factors 45.6 / 35.4 us a sweep, x 6 8.7 / 7.5 us (below 64
+      // slices per SM slices win: x 2 3.6 / 3.8 us)
+      if (S.wide) return true;
+      // rows of up to four entries (units of four slices): in as few rounds as
+      // the ring where the ring's last of at most two is less than 0.72 full:
+      // 7-point 68^3 / 70^3 / 74^3 / 90^3 42.2 / 40.1, 44.3 / 40.4, 45.1 / 42.1
+      // and 72.4 / 68.7 us; with more rounds 78^3 / 100^3 46 / 60 and 80 / 94 us
+      const double units = (S.ns + 3) / 4 * per_warp / 32.0;
+      return S.widest <= 4 && units <= 2.0 && units - std::floor(units) < 0.72 && std::ceil(tiles) <= std::ceil(units);
+    }
+    // FP64 rows of more than ten entries, a second round of slices less than a
+    // quarter full: 27-point 64^3 / 65^3 118.6 / 107.3 and 121.5 / 109.9 us (with
+    // tiles that fill theirs less well 62^3 / 67^3 106.8 / 103.9, 129.1 / 131.7)
+    const double slices = S.ns * per_warp / (S.lanes == 4 ? 32.0 : 48.0);
+    return !T.fp32 && S.widest > 10 && slices > 1.0 && slices < 1.25 && filled(tiles) >= 0.88;
+  }
+  if (!multi) return false;
+  // two columns, and four in FP64, of rows of more than ten entries (more than
+  // a few chunks of gathers per slice): 27-point 130^3 FP64 127 / 104 and 236 /
+  // 206 us a sweep, FP32 two columns 54.7 / 43.4 us; four FP32 columns 66.9 /
+  // 82.9 us
+  if (S.widest > 10 && !(T.fp32 && R == 4)) return true;
+  // two FP64 columns: of short rows (four per lane), where the tiles fill
+  // their rounds: 7-point 70^3 / 90^3 / 104^3 89.6 / 78.4, 160 / 146 and 231 /
+  // 214 us, but 76^3 / 96^3 (0.56 and 0.76 full) 110 / 125 and 190 / 196 us; of
+  // longer ones from 250 slices per SM: cut-cell ILUT 104^3 / 110^3 / 118^3 /
+  // 128^3 422 / 434, 512 / 498, 623 / 596, 767 / 753 us.  Four columns stay on
+  // slices (7-point 104^3 / 110^3 / 128^3 430 / 421, 493 / 536, 762 / 782 us).
+  if (R == 2 && !T.fp32) return T.tile_passes == 4 ? filled(tiles) >= 0.8 : S.widest > 4 && S.ns >= 250 * env.sms;
+  return false;
+}
+
 // Whether a launch on T takes the sliced copy: the default wherever there is
 // one.  An explicit staged shape of A (silu_mat_set_shape, for one column)
 // and, for the factors, an explicit staged variant (2, 3) keep the tiles;
@@ -543,18 +589,7 @@ bool use_slices(silu_ilu F, const DevCsr& T, int R, int ldx) {
   // lanes per row asked for (silu_ilu_set_lanes), where that kernel runs when there are no slices
   const int lanes = &T == &F->dL ? F->lanesL : (&T == &F->dU ? F->lanesU : (&T == &F->A->d ? F->lanesA : 0));
   if (lanes > 0 && T.rp && (R == 1 ? T.ntiles == 0 : !multi_tiles(F, T, R) && !small_block(F, R))) return false;
-  // Large matrices that the tiled sweeps serve faster (per sweep, slices
-  // against tiles):
-  // - FP32, one column, int32 columns (no fewer bytes than the tiles, and no
-  //   ring): 27-point 260 x 260 x 30 factors 45.6 / 35.4 us, x 6 8.7 / 7.5 us
-  //   (below 64 slices per SM slices win: x 2 3.6 / 3.8 us);
-  // - two columns, and four in FP64, of rows of more than ten entries (more
-  //   than a few chunks of gathers per slice): 27-point 130^3 FP64 127 / 104
-  //   and 236 / 206 us, FP32 two columns 54.7 / 43.4 us; four FP32 columns
-  //   66.9 / 82.9 us, and cut-cell 100^3 ILUT rows of ten 44.0 / 44.5 and
-  //   79.8 / 85.6 us.
-  if (R == 1 && T.fp32 && T.sl->wide && T.ntiles > 0 && T.sl->ns >= 64 * F->ctx->env.sms) return false;
-  if (R > 1 && !(T.fp32 && R == 4) && T.sl->widest > 10 && multi_tiles(F, T, R)) return false;
+  if (tiles_faster(T, R, R > 1 && multi_tiles(F, T, R), F->ctx->env)) return false;
   // several columns of an FP32 smoother: only where a kernel that sums in the
   // same order (the tiled multi-column sweep, the fused launch) would run
   // instead: an FP32 sum in another order differs by 1e-7
@@ -1586,7 +1621,7 @@ silu_status silu_mat_residual(silu_mat A, double* r, const double* x, const doub
   if (A->A.n == 0) return SILU_OK;
   cudaStream_t s = ctx->stream;
   try {
-    if (A->d.sliced() && (nrhs > 1 || !A->d.explicit_shape)) {
+    if (A->d.sliced() && (nrhs > 1 || (!A->d.explicit_shape && !silu::tiles_faster(A->d, 1, false, ctx->env)))) {
       for (int c0 = 0; c0 < nrhs;) {
         const int w = slice_width(nrhs - c0);
         LAUNCH(ctx, SILU_K_RESIDUAL, silu::launch_sweep_slices(A->d, silu::MODE_D, ctx->env, w, nrhs, b + c0, x + c0,

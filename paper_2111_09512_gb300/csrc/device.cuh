@@ -215,6 +215,7 @@ cudaError_t launch_sweep_staged(const DevCsr& T, Mode mode, const LaunchEnv& env
 // The staged sweep for R = 2 or 4 interleaved right-hand sides (leading
 // dimension ldx >= R): each staged factor entry feeds R FMAs.  Needs a tile
 // partition with one lane per row (staged_multi_ok); natural row order.
+int tile_warps(bool fp32);  // warps per SM of the tiled sweeps (one tile each at a time)
 bool staged_multi_ok(const DevCsr& T, int R);
 cudaError_t launch_sweep_staged_multi(const DevCsr& T, Mode mode, const LaunchEnv& env, int R, int ldx, const void* c,
                                       const void* in, void* out, const double* dinv, double* x, int epi,

@@ -392,6 +392,8 @@ cudaError_t with_room(silu_ctx ctx, Make make) {
 // The tile entry limit of the automatic launch shape: narrow tiles for FP64
 // values with one lane per row whose rows fit them (silu::narrow_fits).
 int auto_tile_nnz(const Csr& T, bool fp32, int lanes, int passes);
+// Whether R columns on T, which has a sliced copy, are faster on the tiles.
+bool tiles_faster(const DevCsr& T, int R, bool multi, const LaunchEnv& env);
 // Length-sorted copy of T for the staged kernel (silu::make_sorted); clears
 // the copy in d when it would not pay.
 cudaError_t upload_sorted(silu_ctx ctx, const Csr& T, bool fp32, SortedBufs& b, DevCsr& d);

@@ -855,6 +855,8 @@ cudaError_t staged_prepare() {
   return e;
 }
 
+int tile_warps(bool fp32) { return fp32 ? kWarpsF32 : kWarpsF64; }
+
 bool staged_multi_ok(const DevCsr& T, int R) {
   return (R == 2 || R == 4) && T.ntiles > 0 && T.tile_lanes == 1;
 }

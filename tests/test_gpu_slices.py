@@ -298,3 +298,34 @@ def test_columns_at_the_limit_of_16_bits(silu, ctx, span):
         out = dev(np.zeros((n, nrhs)))
         M.residual(out, dev(x), dev(b))
         assert maxabs_err(host(out), oracle.residual(A, x, b)) < FP64_TOL, nrhs
+
+
+# on 152 SMs: 54 to 74 slices per SM, where slices are dealt evenly to the blocks or give way to the tiles
+LINES = [("cutcell7", "ilu0", (64, 65, 63)), ("cutcell7", "ilu0", (71, 70, 69)), ("cutcell7", "ilut", (64, 65, 63)),
+         ("hex27", "ilu0", (65, 64, 65)), ("hex27", "ilu0", (71, 70, 69))]
+
+
+@pytest.mark.parametrize("gen,kind,size", LINES, ids=[f"{g}-{k}-{'x'.join(map(str, s))}" for g, k, s in LINES])
+def test_both_sides_of_the_lines_match_the_lanes_per_row_kernel(silu, ctx, gen, kind, size):
+    """Sums of at most 28 terms of a scaled system, five sweeps: rounding of order 1e-14 (FP32 1e-5)."""
+    A = getattr(synth, gen)(*size, seed=6)
+    n = len(A[0]) - 1
+    M = silu.Matrix(ctx, *A)
+    for nrhs in (1, 2, 3, 4):
+        b, x0 = synth.rhs(n, nrhs, seed=7), synth.rhs(n, nrhs, seed=8)
+        r = dev(np.zeros((n, nrhs)))
+        M.residual(r, dev(x0), dev(b))
+        assert maxabs_err(host(r), oracle.residual(A, x0, b)) < FP64_TOL, nrhs
+    for prec, tol in ((silu.FP64, FP64_TOL), (silu.FP32, 1e-5)):
+        F = silu.ilu_setup(ctx, M, kind, 1e-3, 10, prec=prec)
+        for nrhs in (1, 2, 3, 4):
+            b, x0 = synth.rhs(n, nrhs, seed=7), synth.rhs(n, nrhs, seed=8)
+            out = []
+            for variant, fused in ((0, 0), (1, 1)):
+                F.set_kernel(variant)
+                F.set_fused(fused)
+                x = dev(x0)
+                silu.ilu_smooth(F, x, dev(b), 3, 3)
+                ctx.check()
+                out.append(host(x))
+            assert max(relerr(out[0][:, k], out[1][:, k]) for k in range(nrhs)) < tol, (prec, nrhs)
