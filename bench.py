@@ -103,7 +103,8 @@ def load_peaks():
 
 def sweep_source_hash():
     h = hashlib.sha256()
-    for f in ("slices.cuh", "kernels_slices.cu", "kernels_slices_ring.cu", "sweep_ptx.cuh", "device.cuh"):
+    for f in ("slices.cuh", "kernels_slices.cu", "kernels_slices_ring.cu", "kernels_staged.cu", "bulk.cuh",
+              "sweep_ptx.cuh", "device.cuh"):
         with open(os.path.join(ROOT, "paper_2111_09512_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -128,7 +129,7 @@ def recorded_values(name):
 
 def recorded_traffic():
     """Per-launch DRAM bytes of the sweep kernel on the headline workload."""
-    vals = recorded_values("k_sweep_cutcell128_ilut_traffic.txt")
+    vals = recorded_values("k_slices_cutcell128_ilut_traffic.txt")
     try:
         return float(vals["dram_bytes_per_sweep_launch"]) if vals else None
     except (KeyError, ValueError):
@@ -397,6 +398,10 @@ def run_silu(args):
     padL, padU = (float(v) for v in F.layout()["pad_natural"])
     slots = nL * nnzL * padL + nU * nnzU * padU
     sms = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
+    # what the swept copies hold: 10 bytes per padded entry of the sliced form instead of 12 per entry and the
+    # row pointers, beside the same three vectors
+    sl_bytes = 10 * slots + (nL + nU) * 3 * n * 8
+    streamed = sl_bytes / ((msL + msU) * 1e-3) / 1e9 if msL + msU > 0 else None
     fp64_peak = sms * 2 * (clocks.get("sm_max_mhz") or 2070.0) * 1e6
     fp64_rate = slots / ((msL + msU) * 1e-3) if msL + msU > 0 else None
 
@@ -498,10 +503,14 @@ def run_silu(args):
                        "l2": "inputs larger than L2 (factors + A = %.0f MB > 129 MB)"
                              % ((nnzA * 12 + (nnzL + nnzU) * 12) / 1e6)},
             "hbm_frac_of_" + peak_kind: round(value / world / peak, 4),
-            "roofline": {"bound": "hbm", "kernel": "k_sweep (Richardson sweep SpMV on L_s / Utilde_s)",
+            "roofline": {"bound": "hbm", "kernel": "k_slices (Richardson sweep SpMV on L_s / Utilde_s)",
                          "achieved": round(achieved, 2) if achieved else None, "peak": peak, "unit": "GB/s",
                          "frac": round(achieved / peak, 4) if achieved else None, "peak_kind": peak_kind,
                          "traffic": traffic, "launches": nL + nU,
+                         # achieved counts int32 CSR bytes; this the bytes of the sliced copies that are swept
+                         "streamed_bytes_per_launch": int(sl_bytes / (nL + nU)) if nL + nU else None,
+                         "streamed": round(streamed, 2) if streamed else None,
+                         "streamed_frac": round(streamed / peak, 4) if streamed else None,
                          # consecutive sweeps reuse what L2 holds, so DRAM moves less than the algorithmic
                          # bytes: the DRAM rate is the recorded per-launch traffic over the same mean duration
                          "dram_achieved": round(traffic / ((msL + msU) * 1e-3 / (nL + nU)) / 1e9, 2)
@@ -1489,7 +1498,9 @@ def run_apply_only(args):
                   (direct_trisolve, the automatic schedule) instead of sweeps
       cutcell128_r4: the headline factors with 4 interleaved right-hand sides
       poisson32_r4: 32^3 Poisson ILU(0), 4 interleaved right-hand sides, 5+5
-                  sweeps (a system small enough for the fused application)"""
+                  sweeps (a system small enough for the fused application)
+      hex27_96_fgmres, poisson32_fgmres: 20 FGMRES iterations per step
+                  (27-point 96^3, FP32 factors, 3+3 sweeps; 32^3 Poisson, 5+5)"""
     import torch
     import paper_2111_09512_gb300 as silu
     import synth
@@ -1497,7 +1508,7 @@ def run_apply_only(args):
     stream = torch.cuda.current_stream()
     ctx = silu.Context(0, stream)
     w = args.apply_only
-    direct = False
+    direct, fgmres = False, w.endswith("_fgmres")
     if w in ("cutcell128", "cutcell128_r4"):
         A = synth.cutcell7(EDGE, seed=1)
         kind, prec, mL, mU, vb = "ilut", silu.FP64, ML, MU, 8
@@ -1511,6 +1522,12 @@ def run_apply_only(args):
     elif w == "poisson32_r4":
         A = synth.poisson7(32)
         kind, prec, mL, mU, vb, R = "ilu0", silu.FP64, 5, 5, 8, 4
+    elif w == "hex27_96_fgmres":
+        A = synth.hex27(96, seed=2)
+        kind, prec, mL, mU, vb, R = "ilu0", silu.FP32, 3, 3, 4, 1
+    elif w == "poisson32_fgmres":
+        A = synth.poisson7(32)
+        kind, prec, mL, mU, vb, R = "ilu0", silu.FP64, 5, 5, 8, 1
     else:
         raise SystemExit(f"unknown workload {w}")
     n = len(A[0]) - 1
@@ -1522,7 +1539,10 @@ def run_apply_only(args):
     b = torch.from_numpy(synth.rhs(n, R, seed=1)).cuda()
     x = torch.zeros(n, R, dtype=torch.float64, device="cuda")
     def apply():
-        if direct:
+        if fgmres:
+            x.zero_()
+            silu.fgmres_solve(F, x, b, tol=0.0, restart=30, maxit=20, sweeps_L=mL, sweeps_U=mU)
+        elif direct:
             silu.direct_trisolve(F, x, b)
         else:
             silu.ilu_smooth(F, x, b, mL, mU)
@@ -1551,7 +1571,8 @@ def run_apply_only(args):
         nbytes = (resid_bytes(n, nnzA, R) + (mL - 1) * sweep_bytes(n, st["nnz_L"], R, vb) + 8 * n
                   + (mU - 1) * sweep_bytes(n, st["nnz_U"], R, vb) + 8 * n * R)
     line = {"apply_only": w, "rows": n, "rhs": R, "steps": args.steps, "warmup": args.warmup,
-            "ms_per_application": round(ms, 5), "algorithmic_gbs": round(nbytes / (ms * 1e-3) / 1e9, 1),
+            "ms_per_application": round(ms, 5),
+            "algorithmic_gbs": None if fgmres else round(nbytes / (ms * 1e-3) / 1e9, 1),
             "launches_per_application": {k: v[0] // args.steps for k, v in prof.items() if v[0]},
             "kernel_ms_per_launch": {k: round(v[1] / v[0], 5) for k, v in prof.items() if v[0]}}
     print(json.dumps(line), flush=True)
@@ -1588,7 +1609,8 @@ def main():
     ap.add_argument("--serve-queue", type=int, default=8)
     ap.add_argument("--serve-pool", type=int, default=32)
     ap.add_argument("--apply-only", choices=["cutcell128", "cutcell128_r4", "hex27_256", "hex27_128",
-                                             "hex27_128_direct", "poisson32_r4"], default=None,
+                                             "hex27_128_direct", "poisson32_r4", "hex27_96_fgmres",
+                                             "poisson32_fgmres"], default=None,
                     help="run only smoother applications of one workload (profiling, quick timing)")
     ap.add_argument("--vcycle-only", action="store_true",
                     help="run only V-cycles of the 224^3 GMRES+AMG workload (profiling, quick timing)")

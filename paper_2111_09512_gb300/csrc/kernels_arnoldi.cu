@@ -32,10 +32,16 @@
 // a thread adds its products in row order, a warp by the same shuffle tree, the
 // eight warps of a group one after the other, the np groups as sum_parts adds
 // them.  So results are the bits of the launch-per-vector form.  Two layouts:
-// blocks of GB whole groups, one block per SM, whose reductions pack the trees
-// of a group's eight warps into the lanes of one (9 adds instead of 40); and,
-// for small systems, blocks of half a group (four warps, one per partition),
-// whose warps publish their own sums.
+// k_arnoldi, blocks of one to three whole groups, one block per SM, whose
+// reductions pack the trees of a group's eight warps into the lanes of one (9
+// adds instead of 40); and, for at most 16 groups, k_arnoldi_cluster, one
+// cluster of blocks of a group each, whose warps write their own sums into
+// every block's shared memory (no exchange through L2).
+//
+// Measured per basis vector: the cluster at 16 groups (32^3 rows) 3.0 us, 4.0
+// with a launch per vector, 4.9 with the exchange through L2; 152 to 456 groups
+// of 2048 rows 5.6 to 7.8 us, 8 to 11 with launches; between them the launches
+// (5.0 to 5.8 us with the exchange) are kept.
 #include <cmath>
 
 #include "device.cuh"
