@@ -74,19 +74,19 @@ struct ArnoldiArgs {
 // 0 is an entry that nothing has been written to.
 __host__ __device__ constexpr unsigned exchange_number(int j) { return 1u + (unsigned)j * ((unsigned)j + 3u) / 2u; }
 
-// r[32 q + l] is the value of lane l of warp q (q < 8): the sum over each warp's lanes by
+// r[q] holds lane values of warp q (q < 8): the sum over each warp's lanes by
 // the tree of arn_warp_sum, the trees sharing the lanes of one warp (a lane
 // keeps one value and sends the other to its partner), and those eight sums
 // added one after the other.  Every lane returns the result.
-__device__ __forceinline__ double sum_of_eight_warps(const double* r, int lane) {
-  r += lane;
+__device__ __forceinline__ double sum_of_eight_warps(double (&r)[8], int lane) {
   auto fold = [lane](double a, double b, int off) {  // a's pairs in lanes without bit `off`, b's in the others
     const bool up = (lane & off) != 0;
     const double send = up ? a : b;
     return (up ? b : a) + __shfl_xor_sync(0xffffffffu, send, off);
   };
-  const double t0 = fold(fold(r[0], r[32], 16), fold(r[64], r[96], 16), 8);
-  const double t1 = fold(fold(r[128], r[160], 16), fold(r[192], r[224], 16), 8);
+  const double s0 = fold(r[0], r[1], 16), s1 = fold(r[2], r[3], 16), s2 = fold(r[4], r[5], 16),
+               s3 = fold(r[6], r[7], 16);
+  const double t0 = fold(s0, s1, 8), t1 = fold(s2, s3, 8);
   double v = fold(t0, t1, 4);
   v += __shfl_xor_sync(0xffffffffu, v, 2);
   v += __shfl_xor_sync(0xffffffffu, v, 1);
@@ -134,7 +134,10 @@ __device__ __forceinline__ void givens_column(const ArnoldiArgs& a, double* hc, 
   a.res[1] = q;  // h_{j+1,j}: zero means the Krylov space is exhausted
 }
 
-// One thread's share: rows i0, i0 + S, ..., cnt of them.
+// One thread's share: rows i0, i0 + S, ..., cnt of them.  NARROW: addressed by
+// 32-bit offsets, which spares the registers that three groups per block lack
+// (and costs one or two groups, and the cluster, 1 to 5% of a step).
+template <bool NARROW>
 struct ArnoldiRows {
   unsigned i0, S;
   int cnt;
@@ -145,8 +148,13 @@ struct ArnoldiRows {
     cnt = group < a.np && i0 < (unsigned)a.n ? (int)(((unsigned)a.n - i0 + S - 1) / S) : 0;
   }
   __device__ __forceinline__ void load(const double* p, double (&v)[kArnRows]) const {
+    if constexpr (!NARROW) p += i0;
 #pragma unroll
-    for (int k = 0; k < kArnRows; ++k) v[k] = k < cnt ? p[i0 + (unsigned)k * S] : 0.0;
+    for (int k = 0; k < kArnRows; ++k)
+      if constexpr (NARROW)
+        v[k] = k < cnt ? p[i0 + (unsigned)k * S] : 0.0;
+      else
+        v[k] = k < cnt ? p[(size_t)k * S] : 0.0;
   }
   // this thread's part of <w, v_0>
   __device__ __forceinline__ double first() const {
@@ -173,9 +181,15 @@ struct ArnoldiRows {
   __device__ __forceinline__ void normalize(double h, double* vout) const {
     if (h == 0.0) return;
     const Divider by(h);
+    if constexpr (!NARROW) vout += i0;
 #pragma unroll
     for (int k = 0; k < kArnRows; ++k)
-      if (k < cnt) vout[i0 + (unsigned)k * S] = by(w[k]);
+      if (k < cnt) {
+        if constexpr (NARROW)
+          vout[i0 + (unsigned)k * S] = by(w[k]);
+        else
+          vout[(size_t)k * S] = by(w[k]);
+      }
   }
 };
 
@@ -190,7 +204,7 @@ __global__ void __launch_bounds__(GB * 256, 1) k_arnoldi(ArnoldiArgs a) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int group = blockIdx.x * GB + (threadIdx.x >> 8);
   const bool lead = blockIdx.x == 0;
-  ArnoldiRows rows(a, group, threadIdx.x & 255);
+  ArnoldiRows<GB == 3> rows(a, group, threadIdx.x & 255);
   bool alive = true;
   unsigned tag = a.tag;
   if (lead) load_rotations(a, sh, T);
@@ -199,7 +213,10 @@ __global__ void __launch_bounds__(GB * 256, 1) k_arnoldi(ArnoldiArgs a) {
     lanes[threadIdx.x] = acc;
     __syncthreads();
     if ((warp & 7) == 0) {  // one warp per group
-      const double s = sum_of_eight_warps(lanes + warp * 32, lane);
+      double r[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) r[q] = lanes[(warp + q) * 32 + lane];
+      const double s = sum_of_eight_warps(r, lane);
       if (lane == 0 && group < a.np) publish(a.entries + (step & 1) * a.cap + group, s, tag);
     }
   };
@@ -219,7 +236,10 @@ __global__ void __launch_bounds__(GB * 256, 1) k_arnoldi(ArnoldiArgs a) {
     }
     __syncthreads();
     if (warp == 0) {
-      const double s = sum_of_eight_warps(parts, lane);
+      double r[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) r[q] = parts[q * 32 + lane];
+      const double s = sum_of_eight_warps(r, lane);
       if (lane == 0) total = s;
     }
     __syncthreads();
@@ -260,7 +280,7 @@ __global__ void __launch_bounds__(256, 1) k_arnoldi_cluster(ArnoldiArgs a) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int group = blockIdx.x;  // one cluster: the block's rank
   const bool lead = group == 0;
-  ArnoldiRows rows(a, group, threadIdx.x);
+  ArnoldiRows<false> rows(a, group, threadIdx.x);
   if (lead) load_rotations(a, sh, 256);
   // every block of the cluster runs before another writes into its shared memory
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
