@@ -266,14 +266,16 @@ cudaError_t launch_sweep_slices(const DevCsr& T, Mode mode, const LaunchEnv& env
   if (slices_ring_fits(T, mode, env.sms)) return launch_slices_ring(T, env, c, in, out, dinv, x, epi, s);
   const bool wide = T.sl->wide;
   // Two blocks per SM (beyond eight slices) with the registers of a whole row
-  // leave no room for the launches of other streams.  For rows of up to seven
+  // leave no room for the launches of other streams.  For rows of up to four
   // entries the large matrices' kernel (40 registers) is as fast alone: 7-point
   // ILU(0) 8+8 applications at 36^3 / 40^3 / 42^3 alone 32.5 / 36.9 / 35.8 us
-  // that way, 32.9 / 34.8 / 37.9 us this way, and with eight streams 14.7 /
-  // 18.4 / 22.5 and 14.3 / 14.4 / 14.3 us each.  (ILUT rows of ten at 40^3: 38
-  // us each with eight streams either way.)
+  // that way, 33.3 / 35.8 / 38.2 us this way, and with eight streams 14.7 /
+  // 18.4 / 22.5 and 14.3 / 14.5 / 15.2 us each.  (Rows of seven, the matrix
+  // itself, gain nothing more with streams and cost an FGMRES iteration alone
+  // 2 us; ILUT rows of ten at 40^3 take 38 us each with eight streams either
+  // way.)
   const bool small = !wide && slice_small(T.sl->ns, env.sms) &&
-                     !(mode != MODE_F && T.sl->widest <= 7 && T.sl->ns > kSliceThreads / 32 * env.sms);
+                     !(mode != MODE_F && T.sl->widest <= 4 && T.sl->ns > kSliceThreads / 32 * env.sms);
   // FP32, where the ring does not fit (fewer slices, longer rows, int32
   // columns): a whole row per chunk where rows allow (27-point 32^3 4.5 us a
   // sweep).  Rows of up to four entries at 40 warps per SM and 48 registers:
