@@ -457,10 +457,10 @@ silu_status silu_ilu_set_lanes(silu_ilu F, int lanes_L, int lanes_U, int lanes_A
  * the factor in slices of 32 rows, wherever padding adds at most two fifths
  * to the entries: for one right-hand side with the bits of the staged kernel,
  * for 2 to 4 interleaved ones of an FP64 smoother in column order; without
- * such a copy the staged kernel for one right-hand side, and for 2 or 4 the
- * staged kernel on factors tiled one lane per row when the factor has at
- * least 16 tiles per multiprocessor, the lanes-per-row kernel otherwise),
- * 1 = always the
+ * such a copy, and at sizes and row lengths where it is the faster one, the
+ * staged kernel for one right-hand side, and for 2 or 4 the staged kernel on
+ * factors tiled one lane per row when the factor has at least 16 tiles per
+ * multiprocessor, the lanes-per-row kernel otherwise), 1 = always the
  * lanes-per-row kernel, 2 = the staged kernel wherever it applies, 3 = as 2
  * but on length-sorted copies of the factors for one right-hand side (built
  * on first selection, for the factors where silu_ilu_layout shows sorting
